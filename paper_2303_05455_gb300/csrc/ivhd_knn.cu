@@ -505,7 +505,7 @@ extern "C" ivhd_status ivhd_knn_index_create(const void* X, int32_t dtype, int64
   if (e == cudaSuccess && knn_tc_supported(probe)) {
     const int Kp = knn_tc_kp(dtype, N);
     e = dev_alloc((void**)&idx->B, (size_t)M * Kp * sizeof(__nv_bfloat16), s);
-    if (e == cudaSuccess) e = dev_alloc(&idx->nrm, (size_t)M * 4, s);
+    if (e == cudaSuccess) e = dev_alloc(&idx->nrm, (size_t)(M + 1) * 4, s);
     if (e == cudaSuccess) e = knn_tc_prepare_base(idx->X, dtype, M, N, idx->B, idx->nrm, s);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

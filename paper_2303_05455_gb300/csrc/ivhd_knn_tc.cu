@@ -60,6 +60,8 @@ constexpr int kTStages = 4;
 constexpr int kEpiWarps = 8;  // two warpgroups: each reads one 128-column half of a tile
 constexpr int kTcThreads = 32 * (2 + kEpiWarps);
 constexpr int kMaxKnnSegments = 32;  // column segments of one kNN launch (short query sets)
+constexpr int kGroup = 8;            // columns tested and queued together in the epilogue
+constexpr int kQueue = 14;           // candidates a row holds back before its list takes them
 
 struct KnnSmem {
   static constexpr int a_bytes = kTM * kBK * 2;
@@ -67,7 +69,8 @@ struct KnnSmem {
   static constexpr int stage_bytes = a_bytes + b_bytes;
   static constexpr int bar_offset = kTStages * stage_bytes;
   static constexpr int nrm_offset = bar_offset + 256;  // 8 warps x 128 column terms
-  static constexpr int total = nrm_offset + kEpiWarps * (kTN / 2) * 4 + 1024;  // + slack
+  static constexpr int queue_offset = nrm_offset + kEpiWarps * (kTN / 2) * 4;
+  static constexpr int total = queue_offset + kQueue * 32 * kEpiWarps * 8 + 1024;  // + slack
 };
 
 template <class D>
@@ -75,18 +78,21 @@ __device__ __forceinline__ bool better(D d, int j, D bd, int bj) {
   return d < bd || (d == bd && j < bj);
 }
 
-// Inserts (d, j) into the ascending list (dl, jl) of L entries, dropping the last.
+// Inserts (d, j) into the ascending list (dl, jl) of L entries, dropping the
+// last.  Candidates arrive in increasing j, so an equal key goes behind the
+// ones already listed (the lower index wins the tie) and "<" is the order.
+// Every entry looks at its left neighbour only: no chain of dependent selects.
 template <class D, int L>
 __device__ __forceinline__ void list_insert(D d, int j, D (&dl)[L], int (&jl)[L]) {
 #pragma unroll
-  for (int q = 0; q < L; ++q) {
-    const bool b = better(d, j, dl[q], jl[q]);
-    const D td = dl[q];
-    const int tj = jl[q];
-    dl[q] = b ? d : td;
-    jl[q] = b ? j : tj;
-    d = b ? td : d;
-    j = b ? tj : j;
+  for (int q = L - 1; q > 0; --q) {
+    const bool here = d < dl[q], left = d < dl[q - 1];
+    dl[q] = left ? dl[q - 1] : (here ? d : dl[q]);
+    jl[q] = left ? jl[q - 1] : (here ? j : jl[q]);
+  }
+  if (d < dl[0]) {
+    dl[0] = d;
+    jl[0] = j;
   }
 }
 
@@ -101,14 +107,21 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity,
   return false;
 }
 
+// Twice the certificate's bound over a row's distances: a vertex whose key is
+// above the k-th smallest key by this much or more is not among the k nearest
+// (d_k <= kappa_k + 2 eps max n_j + eps n_i, and d_j >= kappa_j - eps n_i).
+__device__ __forceinline__ float key_slack(float eps_coef, float ni, float n_max) {
+  return 2.f * eps_coef * (ni + n_max);
+}
+
 // U8: exact integer keys; L: list length (kKnnList for float, 8 or kKnnList for uint8).
 template <bool U8, int L>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_knn_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
              const float* __restrict__ nrm_f, const int32_t* __restrict__ nrm_i,
              const float* __restrict__ qnrm_f, const int32_t* __restrict__ qnrm_i, int Mq, int M,
-             int Kp, bool self, int seg_tiles, float eps_coef, int32_t* __restrict__ out_ids,
-             float* __restrict__ out_d, int32_t* __restrict__ err) {
+             int Kp, bool self, int k, int seg_tiles, float eps_coef,
+             int32_t* __restrict__ out_ids, float* __restrict__ out_d, int32_t* __restrict__ err) {
   using D = typename std::conditional<U8, int32_t, float>::type;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -218,9 +231,18 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // (its row quarter) of one 128-column half of each tile: warps 2-5 the
     // first half, warps 6-9 the second, so every row has one list per half.
     // Keys: uint8, the exact distance; float, the lower-bound key
-    // kappa_j = dt_j - eps n_j = n_i + (1 - eps) n_j - 2 <x_i, x_j>~ (see the top).
-    // Columns arrive in increasing j, so a key equal to the list's last never
-    // enters (the earlier index wins the tie) and the test is a plain "<".
+    // kappa_j = dt_j - eps n_j = n_i + (1 - eps) n_j - 2 <x_i, x_j>~ (see the
+    // top); both without n_i, which every key of a row shares, until the end.
+    //
+    // A column is one FMA and one minimum; eight columns share one test against
+    // the row's threshold.  What passes is queued in shared memory (a store per
+    // candidate, whatever the other rows do) and goes to the lists when some row
+    // of the warp has a full queue, all rows together: inserting each candidate
+    // at once made the whole warp walk one row's list, and that, not the tensor
+    // cores, set the time (whole build, 300,000 x 100 floats, k = 5: 70.4 -> 44.2 ms).
+    // uint8: the float key and the float threshold are within 2 of the exact
+    // integers (magnitudes below 2^26), so the test allows 16 and the queue takes
+    // the exact keys.
     constexpr int kHalf = kTN / 2;
     const int quarter = warp & 3;
     const int half = (warp - 2) >> 2;
@@ -228,17 +250,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int i = m0 + r;
     // the half-tile's 128 column terms, staged per warp; each lane prefetches
     // its 4 terms of the next tile into registers while the current one is processed
-    D* nbuf = reinterpret_cast<D*>(smem + KnnSmem::nrm_offset) + (warp - 2) * kHalf;
+    float* nbuf = reinterpret_cast<float*>(smem + KnnSmem::nrm_offset) + (warp - 2) * kHalf;
     constexpr int kPer = kHalf / 32;
+    constexpr int kQueueStride = 32 * kEpiWarps;
+    int2* const queue = reinterpret_cast<int2*>(smem + KnnSmem::queue_offset) + (warp - 2) * 32 + lane;
     const D kMaxKey = U8 ? (D)INT_MAX : (D)__int_as_float(0x7f800000);
+    const float kInf = __int_as_float(0x7f800000);
     const float col_scale = 1.f - eps_coef;
-    D pn[kPer];
+    float pn[kPer];
     auto fetch = [&](int t) {
 #pragma unroll
       for (int e = 0; e < kPer; ++e) {
         const int jc = (t0 + t) * kTN + half * kHalf + e * 32 + lane;
         if constexpr (U8)
-          pn[e] = (jc < M) ? nrm_i[jc] : 0;
+          pn[e] = (jc < M) ? (float)nrm_i[jc] : 0.f;  // at most 2^24: exact
         else
           pn[e] = (jc < M) ? col_scale * nrm_f[jc] : 0.f;
       }
@@ -252,11 +277,44 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     const D ni = (i < Mq) ? (U8 ? (D)qnrm_i[i] : (D)qnrm_f[i]) : (D)0;
     const int iself = self ? i : -1;  // the column a row never lists (self-kNN only)
+    // A candidate is of use only below the list's last key, and below the k-th
+    // key (uint8) or, float, the k-th key plus what separates its distance's
+    // upper bound from a lower bound: slack = 2 eps (n_i + max n_j).
+    const float slack = U8 ? 0.f : key_slack(eps_coef, (float)ni, nrm_f[M]);
+    D thr = kMaxKey;
+    float thr_f = kInf;
+    int held = 0;
+    auto flush = [&]() {
+      const int most = __reduce_max_sync(0xffffffffu, held);
+      for (int q = 0; q < most; ++q) {
+        D d = kMaxKey;
+        int j = INT_MAX;
+        if (q < held) {
+          const int2 e = queue[q * kQueueStride];
+          d = U8 ? (D)e.x : (D)__int_as_float(e.x);
+          j = e.y;
+        }
+        list_insert<D, L>(d, j, dl, jl);
+      }
+      held = 0;
+      D dk = dl[L - 1];  // the k-th key: the smallest from there on
+#pragma unroll
+      for (int q = 0; q < L; ++q)
+        if (q >= k - 1) dk = min(dk, dl[q]);
+      if constexpr (U8) {
+        thr = dk;
+        thr_f = dk == INT_MAX ? kInf : (float)dk + 16.f;
+      } else {
+        thr = fminf(dl[L - 1], dk + slack);
+        thr_f = thr;
+      }
+    };
     bool ok = true;
     fetch(0);
     for (int t = 0; t < n_tiles; ++t) {
       const int b = t & 1;
-      if (!wait_or_abort(&acc_full[b], (t >> 1) & 1, abort_flag)) {
+      if (!wait_or_abort(&acc_full[b], (t >> 1) & 1, abort_flag)) ok = false;
+      if (!__all_sync(0xffffffffu, ok)) {  // the warp stays together below
         ok = false;
         break;
       }
@@ -272,53 +330,44 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         uint32_t v[32];
         tmem_ld32(tbase + c0, v);
         const int jb = n0 + c0;
-        D d[32];
+        float d[32];
 #pragma unroll
         for (int q = 0; q < 32; q += 4) {
-          D nj[4];
-          if constexpr (U8) {
-            const int4 w = *reinterpret_cast<const int4*>(nbuf + c0 + q);
-            nj[0] = w.x, nj[1] = w.y, nj[2] = w.z, nj[3] = w.w;
-          } else {
-            const float4 w = *reinterpret_cast<const float4*>(nbuf + c0 + q);
-            nj[0] = w.x, nj[1] = w.y, nj[2] = w.z, nj[3] = w.w;
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            if constexpr (U8)
-              d[q + e] = ni + nj[e] - 2 * __float2int_rn(__uint_as_float(v[q + e]));
-            else
-              d[q + e] = fmaf(-2.f, __uint_as_float(v[q + e]), ni + nj[e]);
-          }
+          const float4 w = *reinterpret_cast<const float4*>(nbuf + c0 + q);
+          d[q + 0] = fmaf(-2.f, __uint_as_float(v[q + 0]), w.x);
+          d[q + 1] = fmaf(-2.f, __uint_as_float(v[q + 1]), w.y);
+          d[q + 2] = fmaf(-2.f, __uint_as_float(v[q + 2]), w.z);
+          d[q + 3] = fmaf(-2.f, __uint_as_float(v[q + 3]), w.w);
         }
         if (jb + 31 >= M || (jb <= iself && iself <= jb + 31)) {
 #pragma unroll
           for (int q = 0; q < 32; ++q)
-            if (jb + q >= M || jb + q == iself) d[q] = kMaxKey;
+            if (jb + q >= M || jb + q == iself) d[q] = kInf;
         }
-        D mn = d[0];
 #pragma unroll
-        for (int q = 1; q < 32; ++q) mn = min(mn, d[q]);
-        if (mn < dl[L - 1]) {
-          // rare after the first tiles: visit the columns below the threshold in order
-          const D thr = dl[L - 1];
-          uint32_t mask = 0;
-          D tmp[32];
+        for (int g = 0; g < 32; g += kGroup) {
+          float mn = d[g];
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            mask |= (uint32_t)(d[q] < thr) << q;
-            tmp[q] = d[q];
+          for (int q = 1; q < kGroup; ++q) mn = fminf(mn, d[g + q]);
+          if (!__any_sync(0xffffffffu, mn < thr_f)) continue;
+#pragma unroll
+          for (int q = 0; q < kGroup; ++q) {
+            if (d[g + q] < thr_f) {
+              if constexpr (U8) {
+                const int e = (int)nbuf[c0 + g + q] - 2 * __float2int_rn(__uint_as_float(v[g + q]));
+                if (e < thr) queue[held++ * kQueueStride] = make_int2(e, jb + g + q);
+              } else {
+                queue[held++ * kQueueStride] = make_int2(__float_as_int(d[g + q]), jb + g + q);
+              }
+            }
           }
-          while (mask) {
-            const int q = __ffs((int)mask) - 1;
-            mask &= mask - 1;
-            if (tmp[q] < dl[L - 1]) list_insert<D, L>(tmp[q], jb + q, dl, jl);
-          }
+          if (__any_sync(0xffffffffu, held > kQueue - kGroup)) flush();
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
       mbar_arrive(&acc_empty[b]);
     }
+    if (ok) flush();
     if (ok && i < Mq) {
       // the row's list for this segment and half:
       // out_ids / out_key [((i * segments + segment) * 2 + half) * L + q]
@@ -326,10 +375,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
       for (int q = 0; q < L; ++q) {
         out_ids[o + q] = jl[q];
+        const D key = jl[q] == INT_MAX ? kMaxKey : dl[q] + ni;
         if constexpr (U8)
-          reinterpret_cast<int32_t*>(out_d)[o + q] = dl[q];
+          reinterpret_cast<int32_t*>(out_d)[o + q] = key;
         else
-          out_d[o + q] = dl[q];
+          out_d[o + q] = key;
       }
     }
     if (!ok && lane == 0) atomicOr(err, 16);
@@ -370,16 +420,22 @@ __global__ void k_prep_f32(const float* __restrict__ X, int64_t M, int N, int Kp
   if (B) B[e] = b;
 }
 
-// FP32 norms (FP64 sum, rounded once).
+// FP32 norms (FP64 sum, rounded once); the largest goes to nrm[M], which
+// starts at zero (norms are not negative, so their bits order as integers).
 __global__ void k_norms_f32(const float* __restrict__ X, int64_t M, int N, float* __restrict__ nrm) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M) return;
-  double s = 0.0;
-  for (int d = 0; d < N; ++d) {
-    const double x = X[i * N + d];
-    s += x * x;
+  float n = 0.f;
+  if (i < M) {
+    double s = 0.0;
+    for (int d = 0; d < N; ++d) {
+      const double x = X[i * N + d];
+      s += x * x;
+    }
+    n = (float)s;
+    nrm[i] = n;
   }
-  nrm[i] = (float)s;
+  const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(n));
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned*>(nrm + M), top);
 }
 
 // uint8: A = B = x - 128 (zero-padded to Kp); norms of the shifted rows.
@@ -419,10 +475,29 @@ __device__ __forceinline__ void cas(float& d, int& j, int lane, int mask, bool u
   }
 }
 
-// Exact FP32-chain distance of rows i and j (the order of the exact kernel).
+// Exact FP32-chain distance of rows i and j (the order of the exact kernel);
+// vec: both rows start on 16 bytes (N % 4 == 0), four features per load.
 __device__ __forceinline__ float chain_dist(const float* __restrict__ xi,
-                                            const float* __restrict__ xj, int N) {
+                                            const float* __restrict__ xj, int N, bool vec) {
   float acc = 0.f;
+  if (vec) {
+    const float4* a = reinterpret_cast<const float4*>(xi);
+    const float4* b = reinterpret_cast<const float4*>(xj);
+#pragma unroll 4
+    for (int q = 0; q < N / 4; ++q) {
+      const float4 u = a[q], w = b[q];
+      float t = __fsub_rn(u.x, w.x);
+      acc = __fmaf_rn(t, t, acc);
+      t = __fsub_rn(u.y, w.y);
+      acc = __fmaf_rn(t, t, acc);
+      t = __fsub_rn(u.z, w.z);
+      acc = __fmaf_rn(t, t, acc);
+      t = __fsub_rn(u.w, w.w);
+      acc = __fmaf_rn(t, t, acc);
+    }
+    return acc;
+  }
+#pragma unroll 4
   for (int q = 0; q < N; ++q) {
     const float diff = __fsub_rn(xi[q], xj[q]);
     acc = __fmaf_rn(diff, diff, acc);
@@ -438,12 +513,29 @@ __device__ __forceinline__ void warp_sort(float& d, int& j, int lane) {
     for (int m = kk >> 1; m > 0; m >>= 1) cas(d, j, lane, m, (lane & kk) == 0);
 }
 
+// The 32 smallest of a warp's sorted (d, j) and the sorted (dn, jn): the first
+// against the second reversed is bitonic, and a bitonic merge sorts it.
+__device__ __forceinline__ void warp_merge(float& d, int& j, float dn, int jn, int lane) {
+  const float rd = __shfl_sync(0xffffffffu, dn, 31 - lane);
+  const int rj = __shfl_sync(0xffffffffu, jn, 31 - lane);
+  if (better(rd, rj, d, j)) {
+    d = rd;
+    j = rj;
+  }
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) cas(d, j, lane, m, true);
+}
+
 // Warp per row: the row's n_lists candidate lists (two half-tile lists per
-// column segment, L candidates each) are re-ranked by the exact FP32 chain and
-// merged into the 32 best, 32 candidates (one or two lists) per pass, and the
-// row is certified.  A list that is full bounds every vertex it left out by
-// its largest key tau_h (d_ij >= tau_h - eps n_i); a list that is not full
-// left nothing out.
+// column segment, L candidates each) are merged into the 32 smallest keys, and
+// those within the slack of the k-th key are re-ranked by the exact FP32 chain
+// (about eight of 64 at k = 5; re-ranking all of them took 3.25 ms of the
+// 300,000 x 100 build).  When more than 32 are within the slack, all
+// candidates are re-ranked, 32 per pass.
+// Certificate: what a list left out has kappa_j >= min(its largest key if it is
+// full, its k-th key + slack), what was not re-ranked has kappa_j > the
+// merged k-th key + slack; with tau the smallest of these, d_ij >= tau - eps n_i,
+// so the row is final when its exact k-th distance is below that.
 template <int L>
 __global__ void k_rerank(const float* __restrict__ Q, int Mq, const float* __restrict__ X, int M,
                          int N, int k, int n_lists, const int32_t* __restrict__ cand,
@@ -457,47 +549,74 @@ __global__ void k_rerank(const float* __restrict__ Q, int Mq, const float* __res
   const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= Mq) return;
   const float* xi = Q + i * N;
-  float tau = __int_as_float(0x7f800000);
+  const bool vec = N % 4 == 0 && ((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(X)) & 15) == 0;
+  const float inf = __int_as_float(0x7f800000);
+  const float slack = key_slack(eps_coef, qnrm[i], nrm[M]);
+  // L = 32: pass p reads list p; L = 16: lanes 0-15 list 2p, lanes 16-31 list 2p + 1
+  auto entry = [&](int pass) {
+    return (i * n_lists + pass * kPer + ((L == 32) ? 0 : (lane >> 4))) * L + (lane & (L - 1));
+  };
+  auto listed = [&](int j) { return j >= 0 && j < M; };
   float rel = 0.f;
-  float d = __int_as_float(0x7f800000);  // the running 32 best, sorted across the lanes
-  int j = INT_MAX;
+  auto exact = [&](int j, float kj) {
+    const float dc = chain_dist(xi, X + (int64_t)j * N, N, vec);
+    // the approximate distance is the key plus eps n_j
+    rel = fmaxf(rel, fabsf(fmaf(eps_coef, nrm[j], kj) - dc) / fmaxf(qnrm[i] + nrm[j], 1e-30f));
+    return dc;
+  };
+  float tau = inf;
+  float kd = inf;  // the running 32 smallest keys, sorted across the lanes
+  int kj = INT_MAX;
   for (int pass = 0; pass < n_lists / kPer; ++pass) {
-    // L = 32: pass p reads list p; L = 16: lanes 0-15 list 2p, lanes 16-31 list 2p + 1
-    const int h = pass * kPer + ((L == 32) ? 0 : (lane >> 4));
-    const int64_t o = (i * n_lists + h) * L + (lane & (L - 1));
-    const int j0 = cand[o];
-    const float kj = key[o];
-    float dc = __int_as_float(0x7f800000);
-    int jc = INT_MAX;
-    if (j0 >= 0 && j0 < M) {
-      dc = chain_dist(xi, X + (int64_t)j0 * N, N);
-      jc = j0;
-      // the approximate distance is the key plus eps n_j
-      rel = fmaxf(rel, fabsf(fmaf(eps_coef, nrm[j0], kj) - dc) / fmaxf(qnrm[i] + nrm[j0], 1e-30f));
-    }
+    const int64_t o = entry(pass);
+    int j0 = cand[o];
+    float k0 = key[o];
 #pragma unroll
     for (int hh = 0; hh < kPer; ++hh) {
-      // the last entry of each list of this pass
-      const int last = hh * L + L - 1;
-      const int jlast = __shfl_sync(0xffffffffu, j0, last);
-      const float klast = __shfl_sync(0xffffffffu, kj, last);
-      if (jlast >= 0 && jlast < M) tau = fminf(tau, klast);
+      const int last = hh * L + L - 1, kth = hh * L + k - 1;
+      const float klast = __shfl_sync(0xffffffffu, k0, last), kk = __shfl_sync(0xffffffffu, k0, kth);
+      if (listed(__shfl_sync(0xffffffffu, j0, last))) tau = fminf(tau, klast);
+      if (listed(__shfl_sync(0xffffffffu, j0, kth))) tau = fminf(tau, kk + slack);
     }
-    warp_sort(dc, jc, lane);
+    if (!listed(j0)) {
+      k0 = inf;
+      j0 = INT_MAX;
+    }
+    warp_sort(k0, j0, lane);
     if (pass == 0) {
-      d = dc;
-      j = jc;
+      kd = k0;
+      kj = j0;
     } else {
-      // the 32 smallest of two sorted sequences: the running one against the
-      // new one reversed is bitonic, and a bitonic merge sorts it
-      const float rd = __shfl_sync(0xffffffffu, dc, 31 - lane);
-      const int rj = __shfl_sync(0xffffffffu, jc, 31 - lane);
-      if (better(rd, rj, d, j)) {
-        d = rd;
-        j = rj;
+      warp_merge(kd, kj, k0, j0, lane);
+    }
+  }
+  const float bound = __shfl_sync(0xffffffffu, kd, k - 1) + slack;
+  float d = inf;
+  int j = INT_MAX;
+  if (__shfl_sync(0xffffffffu, kd, 31) > bound || !listed(__shfl_sync(0xffffffffu, kj, 31))) {
+    if (listed(kj) && !(kd > bound)) {
+      d = exact(kj, kd);
+      j = kj;
+    }
+    if (listed(__shfl_sync(0xffffffffu, kj, k - 1))) tau = fminf(tau, bound);
+    warp_sort(d, j, lane);
+  } else {
+    for (int pass = 0; pass < n_lists / kPer; ++pass) {
+      const int64_t o = entry(pass);
+      const int j0 = cand[o];
+      float dc = inf;
+      int jc = INT_MAX;
+      if (listed(j0)) {
+        dc = exact(j0, key[o]);
+        jc = j0;
       }
-#pragma unroll
-      for (int m = 16; m > 0; m >>= 1) cas(d, j, lane, m, true);
+      warp_sort(dc, jc, lane);
+      if (pass == 0) {
+        d = dc;
+        j = jc;
+      } else {
+        warp_merge(d, j, dc, jc, lane);
+      }
     }
   }
   float mrel = rel;
@@ -540,7 +659,7 @@ __global__ void k_merge_u8(const int32_t* __restrict__ ids, const int32_t* __res
 template <bool U8, int L>
 cudaError_t launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, const float* nrm_f,
                       const int32_t* nrm_i, const float* qnrm_f, const int32_t* qnrm_i, int Mq,
-                      int M, int Kp, bool self, int segments, int seg_tiles, float eps_coef,
+                      int M, int Kp, bool self, int k, int segments, int seg_tiles, float eps_coef,
                       int32_t* out_ids, float* out_d, int32_t* err, cudaStream_t s) {
   static bool attr_set[64] = {};
   int dev = 0;
@@ -554,8 +673,8 @@ cudaError_t launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, const float*
   }
   const dim3 grid((unsigned)((Mq + kTM - 1) / kTM), (unsigned)segments);
   k_knn_tc<U8, L><<<grid, kTcThreads, KnnSmem::total, s>>>(
-      ma, mb, nrm_f, nrm_i, qnrm_f, qnrm_i, Mq, M, Kp, self, seg_tiles, eps_coef, out_ids, out_d,
-      err);
+      ma, mb, nrm_f, nrm_i, qnrm_f, qnrm_i, Mq, M, Kp, self, k, seg_tiles, eps_coef, out_ids,
+      out_d, err);
   return cudaGetLastError();
 }
 
@@ -598,6 +717,14 @@ int knn_tc_kp(int32_t dtype, int32_t N) {
   return (int)(((K + kBK - 1) / kBK) * kBK);
 }
 
+// The M norms and, at nrm[M], the largest of them.
+static cudaError_t row_norms_f32(const float* X, int64_t M, int N, float* nrm, cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(nrm + M, 0, sizeof(float), s);
+  if (e != cudaSuccess) return e;
+  k_norms_f32<<<(unsigned)((M + 255) / 256), 256, 0, s>>>(X, M, N, nrm);
+  return cudaGetLastError();
+}
+
 cudaError_t knn_tc_prepare_base(const void* X, int32_t dtype, int64_t M, int32_t N,
                                 __nv_bfloat16* B, void* nrm, cudaStream_t s) {
   const int Kp = knn_tc_kp(dtype, N);
@@ -607,7 +734,7 @@ cudaError_t knn_tc_prepare_base(const void* X, int32_t dtype, int64_t M, int32_t
     k_norms_u8s<<<blocks(M), 256, 0, s>>>((const uint8_t*)X, M, N, (int32_t*)nrm);
   } else {
     k_prep_f32<<<blocks(M * Kp), 256, 0, s>>>((const float*)X, M, N, Kp, nullptr, B);
-    k_norms_f32<<<blocks(M), 256, 0, s>>>((const float*)X, M, N, (float*)nrm);
+    return row_norms_f32((const float*)X, M, N, (float*)nrm, s);
   }
   return cudaGetLastError();
 }
@@ -677,10 +804,10 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
         k_norms_u8s<<<blocks(Mq), 256, 0, s>>>(Q, Mq, N, qnrm);
       }
       e = (L == 8) ? launch_tc<true, 8>(ma, mb, nullptr, nrm, nullptr, qnrm, (int)Mq, (int)M, Kp,
-                                        P.self, segs, seg_tiles, 0.f, lids, (float*)lkeys, err,
+                                        P.self, k, segs, seg_tiles, 0.f, lids, (float*)lkeys, err,
                                         s)
                    : launch_tc<true, kKnnList>(ma, mb, nullptr, nrm, nullptr, qnrm, (int)Mq,
-                                               (int)M, Kp, P.self, segs, seg_tiles, 0.f, lids,
+                                               (int)M, Kp, P.self, k, segs, seg_tiles, 0.f, lids,
                                                (float*)lkeys, err, s);
     }
     if (e == cudaSuccess) {
@@ -691,8 +818,8 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
       e = cudaGetLastError();
     }
   } else {
-    float* nrm = base ? (float*)const_cast<void*>(base->nrm) : b.get<float>(M);
-    float* qnrm = P.self ? nrm : b.get<float>(Mq);
+    float* nrm = base ? (float*)const_cast<void*>(base->nrm) : b.get<float>(M + 1);
+    float* qnrm = P.self ? nrm : b.get<float>(Mq + 1);
     const int L = (k <= 8) ? 16 : kKnnList;  // candidates per row and half
     int32_t* cand = b.get<int32_t>(Mq * n_lists * L);
     float* cd = b.get<float>(Mq * n_lists * L);
@@ -706,13 +833,15 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
       } else {
         if (!base) k_prep_f32<<<blocks(M * Kp), 256, 0, s>>>(X, M, N, Kp, nullptr, B);
         k_prep_f32<<<blocks(Mq * Kp), 256, 0, s>>>(Q, Mq, N, Kp, A, nullptr);
-        k_norms_f32<<<blocks(Mq), 256, 0, s>>>(Q, Mq, N, qnrm);
+        e = row_norms_f32(Q, Mq, N, qnrm, s);
       }
-      if (!base) k_norms_f32<<<blocks(M), 256, 0, s>>>(X, M, N, nrm);
+      if (!base && e == cudaSuccess) e = row_norms_f32(X, M, N, nrm, s);
+    }
+    if (e == cudaSuccess) {
       e = (L == 16) ? launch_tc<false, 16>(ma, mb, nrm, nullptr, qnrm, nullptr, (int)Mq, (int)M,
-                                           Kp, P.self, segs, seg_tiles, eps_coef, cand, cd, err, s)
+                                           Kp, P.self, k, segs, seg_tiles, eps_coef, cand, cd, err, s)
                     : launch_tc<false, kKnnList>(ma, mb, nrm, nullptr, qnrm, nullptr, (int)Mq,
-                                                 (int)M, Kp, P.self, segs, seg_tiles, eps_coef,
+                                                 (int)M, Kp, P.self, k, segs, seg_tiles, eps_coef,
                                                  cand, cd, err, s);
     }
     if (e == cudaSuccess) {

@@ -36,15 +36,15 @@ struct KnnProblem {
 bool knn_tc_supported(const KnnProblem& P);
 
 // A base set prepared once for many queries: its BF16 operand (M x Kp, the
-// layout knn_tc_build makes) and its row norms (float for float data, int32
-// norms of the rows shifted by -128 for uint8).
+// layout knn_tc_build makes) and its row norms (float for float data, followed by
+// the largest of them; int32 norms of the rows shifted by -128 for uint8).
 struct KnnBase {
   const __nv_bfloat16* B;
   const void* nrm;
 };
 // Padded GEMM depth of the operands (K = N for uint8, 3N for float).
 int knn_tc_kp(int32_t dtype, int32_t N);
-// Fills B (M x knn_tc_kp) and nrm (M) for the base set X; stream-ordered.
+// Fills B (M x knn_tc_kp) and nrm (M + 1) for the base set X; stream-ordered.
 cudaError_t knn_tc_prepare_base(const void* X, int32_t dtype, int64_t M, int32_t N,
                                 __nv_bfloat16* B, void* nrm, cudaStream_t s);
 
