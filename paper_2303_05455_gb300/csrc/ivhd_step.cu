@@ -785,127 +785,321 @@ __device__ __forceinline__ void cluster_store(uint32_t addr, float2 v) {
                : "memory");
 }
 
-template <int MODE, int METRIC>
-__global__ void __launch_bounds__(kResidentThreads, 1) k_cluster(const StepArgs A, int64_t n_iter) {
+// The force on one row from its first 4 G entries, held in registers and
+// gathered from shared memory, in the order and with the values of rvisit8 /
+// rvisit4.  any_rn has bit q set when some lane of the warp holds a
+// random-neighbour term at q: groups of four without one skip the square roots.
+constexpr int kHeld = 16;
+constexpr int kHeldThreads = 1024;  // 64 registers a thread
+template <int METRIC, int G>
+__device__ __forceinline__ void held_forces(const uint32_t (&e)[kHeld], uint32_t any_rn,
+                                            const float2* src, float2 yi, float c, float& fx,
+                                            float& fy) {
+  float2 g[4 * G];
+#pragma unroll
+  for (int q = 0; q < 4 * G; ++q) g[q] = src[e[q] & kIdxMask];
+#pragma unroll
+  for (int t = 0; t < G; ++t) {
+    if constexpr (METRIC == IVHD_METRIC_L2) {
+      float ux[4], uy[4], w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        ux[q] = g[4 * t + q].x - yi.x;
+        uy[q] = g[4 * t + q].y - yi.y;
+        w[q] = (e[4 * t + q] & kW2Bit) ? 2.f : 1.f;
+      }
+      if ((any_rn >> (4 * t)) & 15u) {
+        // the four square roots side by side: a warp alone on its scheduler
+        // waits for each otherwise
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float d2 = fmaf(uy[q], uy[q], ux[q] * ux[q]);
+          const float wr = (d2 > 0.f) ? c * (1.f - rsqrtf(d2)) : 0.f;
+          w[q] = (e[4 * t + q] & kRnBit) ? wr : w[q];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        fx = fmaf(w[q], ux[q], fx);
+        fy = fmaf(w[q], uy[q], fy);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        force_term<METRIC>(e[4 * t + q], g[4 * t + q], yi, c, fx, fy);
+    }
+  }
+}
+
+// Store of a position into block `rank` of the cluster, whose barrier there
+// counts the bytes once they have landed.
+__device__ __forceinline__ void cluster_store_async(uint32_t addr, uint32_t bar, uint32_t rank,
+                                                    float2 v) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+                   cluster_map(addr, rank)),
+               "f"(v.x), "f"(v.y), "r"(cluster_map(bar, rank))
+               : "memory");
+}
+// Bounded wait for a phase of this block's barrier (every poll may itself
+// suspend the thread for a while): false when it did not complete.
+constexpr int kClusterPolls = 1 << 20;
+__device__ __forceinline__ bool cluster_wait(uint32_t bar, uint32_t parity) {
+  for (int it = 0; it < kClusterPolls; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.b32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// A row of a work item: its int4 groups for this lane are at[l], at[l + g], ...
+struct ClusterRow {
+  const int4* at;
+  int p, l, g, ng;
+  bool own;
+};
+__device__ __forceinline__ ClusterRow cluster_row(const StepArgs& A, int item, int lane) {
+  ClusterRow R{nullptr, 0, 0, 32, 0, false};
+  if (item < A.hub_warps) {
+    const HubSlot h = hub_slot(item, lane, A.n_full, A.mid_g);
+    const bool valid = h.row < A.n_hub;
+    R.p = valid ? h.row : 0;
+    R.l = h.l;
+    R.g = h.g;
+    R.own = valid && h.l == 0;
+    if (valid) {
+      const int beg = A.hub_off[R.p], end = A.hub_off[R.p + 1];
+      R.at = reinterpret_cast<const int4*>(A.ids + beg);
+      R.ng = row_ok(beg, end, A.n_slots) ? (end - beg) >> 2 : 0;
+    }
+  } else {
+    const int sl = item - A.hub_warps;
+    const int p = A.n_hub + sl * 32 + lane;
+    R.own = p < A.M;
+    R.p = R.own ? p : 0;
+    // lane l reads group g at [g * 32 + l]: the slice's rows side by side
+    const int64_t beg = A.slice_off[sl];
+    R.at = reinterpret_cast<const int4*>(A.ids + beg) + lane;
+    R.ng = row_ok(beg, beg + (int64_t)A.slice_w[sl] * 128, A.n_slots) ? A.slice_w[sl] * 32 : 0;
+  }
+  return R;
+}
+
+// One update of a vertex at ym with state (v, ex); returns the new position.
+template <int MODE>
+__device__ __forceinline__ float2 cluster_update(const StepArgs& A, float fx, float fy, float2 ym,
+                                                 float2& v, float2& ex) {
+  float2 vn, yn;
+  if (MODE == kMomentum) {
+    momentum_update(A.a, A.b, fx, fy, ym, v, vn, yn);
+    v = vn;
+  } else if (MODE == kNesterov) {
+    nesterov_update(A.a, A.b, fx, fy, ym, v, vn, yn);
+    v = vn;
+  } else {
+    adadelta_update(A.rho, A.eps, fx, fy, ym, v, ex, yn);
+  }
+  return yn;
+}
+
+// HELD: every block has a warp for each of its items and every lane's part of
+// a row fits kHeld entries (hub threshold at most 16), so a warp keeps its item
+// for the whole call: entries, the owner's position and its optimiser state
+// stay in registers, and a step reads nothing but the gathered positions from
+// shared memory.  Steps are separated by byte-counting barriers: a position is
+// stored asynchronously into every block, and a block goes on once all M have
+// arrived.  That also means every warp of the cluster is done gathering, so
+// two buffers (and a barrier for each) suffice.
+// What bounds it: the broadcast.  A block sends 8 M bytes a step through its
+// distributed-shared-memory port at about 16 bytes per clock, whatever the
+// cluster's size; store, arrival and wait alone take 0.54 us at 2,048 vertices
+// (0.20 us with 32 stores), and a cluster barrier after the same stores (a
+// release of every warp's remote stores) 1.03 us.  Per step,
+// k = 2, r = 1: 2,000 vertices 2.01 -> 1.17 us, 4,000 2.49 -> 2.05 us; k = 5,
+// 2,000 vertices 3.13 -> 2.37 us (before: ids read every step, through an L1 that
+// the barrier had emptied).
+// A wait that runs out (bounded) ends the call with NaN positions, which
+// ivhd_stress reports.
+//
+// Otherwise (custom layout shapes, more items) the warps loop over the items,
+// read offsets and ids every step, and a cluster barrier separates the steps.
+template <int MODE, int METRIC, bool HELD>
+__global__ void __launch_bounds__(HELD ? kHeldThreads : kResidentThreads, 1)
+    k_cluster(const StepArgs A, int64_t n_iter) {
   extern __shared__ __align__(16) unsigned char rsm[];
   const int M = A.M, Mp = (A.M + 1) & ~1;
   float2* ys0 = reinterpret_cast<float2*>(rsm);
   float2* ys1 = ys0 + Mp;
-  float2* vs = ys1 + Mp;
-  float2* es = vs + Mp;  // Adadelta E[dx^2]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = (int)(blockDim.x >> 5);
   const uint32_t rank = cluster_rank();
   const int n_items = A.hub_warps + A.n_slices;
   const int it_lo = (int)((int64_t)n_items * rank / kClusterCTAs);
   const int it_hi = (int)((int64_t)n_items * (rank + 1) / kClusterCTAs);
-  // the first vertex of an item: items cover contiguous, ascending vertex ranges
-  auto first_vertex = [&](int item) {
-    if (item < A.n_full) return item;
-    if (item < A.hub_warps) return A.n_full + (item - A.n_full) * (32 / A.mid_g);
-    return A.n_hub + (item - A.hub_warps) * 32;
-  };
-  const int v_lo = min(M, first_vertex(it_lo)), v_hi = min(M, first_vertex(it_hi));
-
-  for (int p = threadIdx.x; p < M; p += blockDim.x) ys0[p] = A.y[A.cur][p];
-  for (int p = v_lo + threadIdx.x; p < v_hi; p += blockDim.x) {
-    vs[p] = A.v[0][p];
-    if (MODE == kAdadelta) es[p] = A.s2[p];
-  }
-  // every block's copy is loaded before any block writes into it
-  cluster_barrier();
   const uint32_t a0 = (uint32_t)__cvta_generic_to_shared(ys0);
   const uint32_t a1 = (uint32_t)__cvta_generic_to_shared(ys1);
-
-  for (int64_t it = 0; it < n_iter; ++it) {
-    const float2* src = (it & 1) ? ys1 : ys0;
-    const uint32_t dst_a = (it & 1) ? a0 : a1;
-    for (int item = it_lo + warp; item < it_hi; item += nwarps) {
-      float fx = 0.f, fy = 0.f;
-      float2 ym = make_float2(0.f, 0.f);
-      int p;
-      bool own;
-      if (item < A.hub_warps) {
-        const HubSlot h = hub_slot(item, lane, A.n_full, A.mid_g);
-        const bool valid = h.row < A.n_hub;
-        int ng = 0;
-        const int4* row = nullptr;
-        p = h.row;
-        if (valid) {
-          ym = src[p];
-          const int beg = A.hub_off[p], end = A.hub_off[p + 1];
-          row = reinterpret_cast<const int4*>(A.ids + beg);
-          ng = row_ok(beg, end, A.n_slots) ? (end - beg) >> 2 : 0;
-        }
-        int g = h.l;
-        for (; g + h.g < ng; g += 2 * h.g)
-          rvisit8<MODE, METRIC>(row[g], row[g + h.g], src, (uint32_t)M, ym, A.c, fx, fy);
-        if (g < ng) rvisit4<MODE, METRIC>(row[g], src, (uint32_t)M, ym, A.c, fx, fy);
-        group_sum(fx, fy, h.g);
-        own = valid && h.l == 0;
-      } else {
-        const int sl = item - A.hub_warps;
-        p = A.n_hub + sl * 32 + lane;
-        own = p < M;
-        if (own) ym = src[p];
-        const int4* base = reinterpret_cast<const int4*>(A.ids + A.slice_off[sl]) + lane;
-        const int W =
-            row_ok(A.slice_off[sl], A.slice_off[sl] + (int64_t)A.slice_w[sl] * 128, A.n_slots)
-                ? A.slice_w[sl]
-                : 0;
-        int g = 0;
-        for (; g + 1 < W; g += 2)
-          rvisit8<MODE, METRIC>(base[g * 32], base[(g + 1) * 32], src, (uint32_t)M, ym, A.c, fx,
-                                fy);
-        if (g < W) rvisit4<MODE, METRIC>(base[g * 32], src, (uint32_t)M, ym, A.c, fx, fy);
-      }
-      if (!own) continue;
-      float2 yn;
-      if (MODE == kMomentum) {
-        float2 vn;
-        momentum_update(A.a, A.b, fx, fy, ym, vs[p], vn, yn);
-        vs[p] = vn;
-      } else if (MODE == kNesterov) {
-        float2 vn;
-        nesterov_update(A.a, A.b, fx, fy, ym, vs[p], vn, yn);
-        vs[p] = vn;
-      } else {
-        float2 eg = vs[p], ex = es[p];
-        adadelta_update(A.rho, A.eps, fx, fy, ym, eg, ex, yn);
-        vs[p] = eg;
-        es[p] = ex;
-      }
-      const uint32_t off = dst_a + (uint32_t)p * (uint32_t)sizeof(float2);
-#pragma unroll
-      for (int r = 0; r < kClusterCTAs; ++r) cluster_store(cluster_map(off, (uint32_t)r), yn);
-    }
-    cluster_barrier();
-  }
-  const float2* fin = (n_iter & 1) ? ys1 : ys0;
   float2* yout = A.y[A.cur ^ (int)(n_iter & 1)];
-  for (int p = v_lo + threadIdx.x; p < v_hi; p += blockDim.x) {
-    yout[p] = fin[p];
-    A.v[0][p] = vs[p];
-    if (MODE == kAdadelta) A.s2[p] = es[p];
+
+  for (int p = threadIdx.x; p < M; p += blockDim.x) ys0[p] = A.y[A.cur][p];
+
+  if constexpr (HELD) {
+    __shared__ __align__(8) uint64_t bars[2];
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bars);
+    if (threadIdx.x == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const int item = it_lo + warp;
+    const bool busy = item < it_hi;
+    const bool hub = item < A.hub_warps;
+    ClusterRow R{nullptr, 0, 0, 32, 0, false};
+    uint32_t e[kHeld];
+    uint32_t any_rn = 0;
+    int groups = 0;
+    float2 v = make_float2(0.f, 0.f), ex = v;
+    if (busy) {
+      R = cluster_row(A, item, lane);
+#pragma unroll
+      for (int t = 0; t < kHeld / 4; ++t) {
+        const int at = R.l + t * R.g;
+        const int4 w = at < R.ng ? R.at[at] : make_int4(-1, -1, -1, -1);
+        e[4 * t] = (uint32_t)w.x;
+        e[4 * t + 1] = (uint32_t)w.y;
+        e[4 * t + 2] = (uint32_t)w.z;
+        e[4 * t + 3] = (uint32_t)w.w;
+        groups += __any_sync(0xffffffffu, at < R.ng);
+      }
+#pragma unroll
+      for (int q = 0; q < kHeld; ++q) {
+        // padding gathers the row's own position as an nn term: u = 0, no force
+        if (e[q] == kPad || !index_ok(e[q] & kIdxMask, (uint32_t)M)) e[q] = (uint32_t)R.p;
+        any_rn |= (uint32_t)(__any_sync(0xffffffffu, (e[q] & kRnBit) != 0)) << q;
+      }
+      if (R.own) {
+        v = A.v[0][R.p];
+        if (MODE == kAdadelta) ex = A.s2[R.p];
+      }
+    }
+    // every block's copy is loaded, and its barriers are set up, before any
+    // block stores into it
+    cluster_barrier();
+    float2 ym = ys0[R.p];
+    bool ok = true;
+    for (int64_t it = 0; it < n_iter; ++it) {
+      const uint32_t b = bar + (uint32_t)(it & 1) * 8u;
+      if (threadIdx.x == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b),
+                     "r"((uint32_t)M * 8u)
+                     : "memory");
+      if (busy) {
+        const float2* src = (it & 1) ? ys1 : ys0;
+        float fx = 0.f, fy = 0.f;
+        if (groups == 2)
+          held_forces<METRIC, 2>(e, any_rn, src, ym, A.c, fx, fy);
+        else if (groups == 1)
+          held_forces<METRIC, 1>(e, any_rn, src, ym, A.c, fx, fy);
+        else if (groups == 3)
+          held_forces<METRIC, 3>(e, any_rn, src, ym, A.c, fx, fy);
+        else if (groups == 4)
+          held_forces<METRIC, 4>(e, any_rn, src, ym, A.c, fx, fy);
+        if (hub) group_sum(fx, fy, R.g);
+        ym = cluster_update<MODE>(A, fx, fy, ym, v, ex);
+        if (R.own) {
+          const uint32_t to = ((it & 1) ? a0 : a1) + (uint32_t)R.p * 8u;
+#pragma unroll
+          for (uint32_t r = 0; r < kClusterCTAs; ++r)
+            cluster_store_async(to, b, (rank + r) % kClusterCTAs, ym);
+        }
+        if (hub) {
+          // the lanes of a hub row take the owner's position
+          ym.x = __shfl_sync(0xffffffffu, ym.x, lane & ~(R.g - 1));
+          ym.y = __shfl_sync(0xffffffffu, ym.y, lane & ~(R.g - 1));
+        }
+      }
+      ok = __all_sync(0xffffffffu, cluster_wait(b, (uint32_t)(it >> 1) & 1u));
+      if (!ok) break;
+    }
+    if (R.own) {
+      const float nan = __int_as_float(0x7fffffff);
+      yout[R.p] = ok ? ym : make_float2(nan, nan);
+      A.v[0][R.p] = v;
+      if (MODE == kAdadelta) A.s2[R.p] = ex;
+    }
+  } else {
+    float2* vs = ys1 + Mp;
+    float2* es = vs + Mp;  // Adadelta E[dx^2]
+    const int nwarps = (int)(blockDim.x >> 5);
+    // the first vertex of an item: items cover contiguous, ascending vertex ranges
+    auto first_vertex = [&](int item) {
+      if (item < A.n_full) return item;
+      if (item < A.hub_warps) return A.n_full + (item - A.n_full) * (32 / A.mid_g);
+      return A.n_hub + (item - A.hub_warps) * 32;
+    };
+    const int v_lo = min(M, first_vertex(it_lo)), v_hi = min(M, first_vertex(it_hi));
+    for (int p = v_lo + threadIdx.x; p < v_hi; p += blockDim.x) {
+      vs[p] = A.v[0][p];
+      if (MODE == kAdadelta) es[p] = A.s2[p];
+    }
+    // every block's copy is loaded before any block writes into it
+    cluster_barrier();
+    for (int64_t it = 0; it < n_iter; ++it) {
+      const float2* src = (it & 1) ? ys1 : ys0;
+      const uint32_t dst_a = (it & 1) ? a0 : a1;
+      for (int item = it_lo + warp; item < it_hi; item += nwarps) {
+        const ClusterRow R = cluster_row(A, item, lane);
+        const float2 ym = src[R.p];
+        float fx = 0.f, fy = 0.f;
+        int g = R.l;
+        for (; g + R.g < R.ng; g += 2 * R.g)
+          rvisit8<MODE, METRIC>(R.at[g], R.at[g + R.g], src, (uint32_t)M, ym, A.c, fx, fy);
+        if (g < R.ng) rvisit4<MODE, METRIC>(R.at[g], src, (uint32_t)M, ym, A.c, fx, fy);
+        if (item < A.hub_warps) group_sum(fx, fy, R.g);
+        if (!R.own) continue;
+        float2 v = vs[R.p], ex = MODE == kAdadelta ? es[R.p] : v;
+        const float2 yn = cluster_update<MODE>(A, fx, fy, ym, v, ex);
+        vs[R.p] = v;
+        if (MODE == kAdadelta) es[R.p] = ex;
+        const uint32_t off = dst_a + (uint32_t)R.p * (uint32_t)sizeof(float2);
+#pragma unroll
+        for (int r = 0; r < kClusterCTAs; ++r) cluster_store(cluster_map(off, (uint32_t)r), yn);
+      }
+      cluster_barrier();
+    }
+    const float2* fin = (n_iter & 1) ? ys1 : ys0;
+    for (int p = v_lo + threadIdx.x; p < v_hi; p += blockDim.x) {
+      yout[p] = fin[p];
+      A.v[0][p] = vs[p];
+      if (MODE == kAdadelta) A.s2[p] = es[p];
+    }
   }
   // no block leaves while a peer could still address its shared memory
   cluster_barrier();
 }
 
-template <int MODE, int METRIC>
-static cudaError_t launch_cl(const StepArgs& A, int64_t n_iter, size_t smem, cudaStream_t s) {
+template <int MODE, int METRIC, bool HELD>
+static cudaError_t launch_cl(const StepArgs& A, int64_t n_iter, size_t smem, int threads,
+                             cudaStream_t s) {
   static bool attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_cluster<MODE, METRIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem);
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_cluster<MODE, METRIC, HELD>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kClusterCTAs);
-  cfg.blockDim = dim3(kResidentThreads);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -915,7 +1109,19 @@ static cudaError_t launch_cl(const StepArgs& A, int64_t n_iter, size_t smem, cud
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_cluster<MODE, METRIC>, A, n_iter);
+  return cudaLaunchKernelEx(&cfg, k_cluster<MODE, METRIC, HELD>, A, n_iter);
+}
+
+// A warp per item where a block has warps enough for its items and no lane has
+// more than kHeld entries of a row: SELL rows are shorter than the hub
+// threshold, hub rows shorter than 512 / vpw entries on 32 / vpw lanes.
+template <int MODE, int METRIC>
+static cudaError_t launch_cl(const StepArgs& A, int hub_threshold, int64_t n_iter, size_t smem,
+                             cudaStream_t s) {
+  const int items = (A.hub_warps + A.n_slices + kClusterCTAs - 1) / kClusterCTAs;
+  return items <= kHeldThreads / 32 && hub_threshold <= kHeld
+             ? launch_cl<MODE, METRIC, true>(A, n_iter, smem, 32 * items, s)
+             : launch_cl<MODE, METRIC, false>(A, n_iter, smem, kResidentThreads, s);
 }
 
 // Shared memory of the resident kernel with and without the id rows.
@@ -1019,14 +1225,14 @@ cudaError_t launch_resident(ivhd_ctx* ctx, int64_t n_iter, cudaStream_t s) {
   if (mode == 3) {
     switch (ctx->p.opt) {
       case IVHD_OPT_NESTEROV:
-        return l1 ? launch_cl<kNesterov, IVHD_METRIC_L1>(A, n_iter, smem, s)
-                  : launch_cl<kNesterov, IVHD_METRIC_L2>(A, n_iter, smem, s);
+        return l1 ? launch_cl<kNesterov, IVHD_METRIC_L1>(A, ctx->hub_threshold, n_iter, smem, s)
+                  : launch_cl<kNesterov, IVHD_METRIC_L2>(A, ctx->hub_threshold, n_iter, smem, s);
       case IVHD_OPT_ADADELTA:
-        return l1 ? launch_cl<kAdadelta, IVHD_METRIC_L1>(A, n_iter, smem, s)
-                  : launch_cl<kAdadelta, IVHD_METRIC_L2>(A, n_iter, smem, s);
+        return l1 ? launch_cl<kAdadelta, IVHD_METRIC_L1>(A, ctx->hub_threshold, n_iter, smem, s)
+                  : launch_cl<kAdadelta, IVHD_METRIC_L2>(A, ctx->hub_threshold, n_iter, smem, s);
       default:
-        return l1 ? launch_cl<kMomentum, IVHD_METRIC_L1>(A, n_iter, smem, s)
-                  : launch_cl<kMomentum, IVHD_METRIC_L2>(A, n_iter, smem, s);
+        return l1 ? launch_cl<kMomentum, IVHD_METRIC_L1>(A, ctx->hub_threshold, n_iter, smem, s)
+                  : launch_cl<kMomentum, IVHD_METRIC_L2>(A, ctx->hub_threshold, n_iter, smem, s);
     }
   }
   switch (ctx->p.opt) {
