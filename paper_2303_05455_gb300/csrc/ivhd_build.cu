@@ -876,6 +876,7 @@ ivhd_status build_layout(ivhd_ctx* ctx, bool draw_rn, uint64_t rn_epoch) {
   }
   IVHD_TRY(cudaGetLastError());
   // the layout is complete once the stream reaches here; scratch frees follow in order
+  ctx->layout_fresh = true;
   return IVHD_OK;
 }
 

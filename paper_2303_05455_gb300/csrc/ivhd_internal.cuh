@@ -194,6 +194,7 @@ struct ivhd_ctx {
   int32_t* hub_off = nullptr;
   int32_t* slice_off = nullptr;
   int32_t* slice_w = nullptr;
+  bool layout_fresh = false;  // built since the last step launched outside a graph
   int64_t n_slots = 0, n_hub = 0, n_slices = 0;
   int64_t n_ge[3] = {0, 0, 0};  // rows with at least 256, 128, 64 entries (all hub rows)
   int64_t n_wide = 0;           // hub rows with at least kWideRow entries (kWideWarps warps each)

@@ -551,6 +551,140 @@ __global__ void __maxnreg__(step_max_regs<MODE>()) k_step(const StepArgs A) {
   step_block<MODE, POS, METRIC, ADAPT, true>(A, (int)blockIdx.x, cur);
 }
 
+// The step for graphs whose whole grid fits the GPU beside the next one's: a
+// step there is a chain of waits (launch, row offsets, ids, gathers, store), not
+// traffic.  The layout is never written by a step, so a block reads its rows'
+// offsets and first kPre id groups per lane before it waits for the previous
+// grid, and lets the next grid launch as soon as that wait is over: the next
+// blocks are resident, with their ids in registers, while this grid gathers.
+// Traversal and arithmetic are those of k_step.
+constexpr int kPre = 4;  // id groups held per lane
+template <int MODE, int POS, int METRIC>
+__global__ void __launch_bounds__(kMaxStepBlock) k_step_ahead(const StepArgs A) {
+  const int lane = threadIdx.x & 31;
+  const int wib = threadIdx.x >> 5;
+  const int vb = (int)blockIdx.x;
+  // this lane's groups are row[l], row[l + g], ... below ng; p: its vertex
+  const int4* row = nullptr;
+  int l = 0, g = 32, ng = 0, p = -1;
+  bool own = false;
+  const bool wide = vb < A.nb_wide;
+  const int grp = wib / kWideWarps;
+  if (wide) {
+    const int r = vb * (A.wpb / kWideWarps) + grp;
+    l = (int)threadIdx.x - grp * kWideWarps * 32;
+    g = kWideWarps * 32;
+    if (r < A.n_wide) {
+      p = r;
+      own = l == 0;
+    }
+  } else if (vb < A.nb_wide + A.nb_hub) {
+    const int w = (vb - A.nb_wide) * A.wpb + wib;
+    if (w < A.hub_warps) {
+      const HubSlot h = hub_slot(w, lane, A.n_full, A.mid_g);
+      l = h.l;
+      g = h.g;
+      if (A.n_wide + h.row < A.n_hub) {
+        p = A.n_wide + h.row;
+        own = l == 0;
+      }
+    }
+  }
+  const bool hub = vb < A.nb_wide + A.nb_hub;
+  if (hub) {
+    if (p >= 0) {
+      const int beg = __ldg(A.hub_off + p), end = __ldg(A.hub_off + p + 1);
+      row = reinterpret_cast<const int4*>(A.ids + beg);
+      ng = row_ok(beg, end, A.n_slots) ? (end - beg) >> 2 : 0;
+    }
+  } else {
+    const int s = (vb - A.nb_wide - A.nb_hub) * A.wpb + wib;
+    if (s < A.n_slices) {
+      p = A.n_hub + s * 32 + lane;
+      own = p < A.M;
+      const int64_t beg = __ldg(A.slice_off + s);
+      const int W = __ldg(A.slice_w + s);
+      row = reinterpret_cast<const int4*>(A.ids + beg) + lane;
+      ng = row_ok(beg, beg + (int64_t)W * 128, A.n_slots) ? W * 32 : 0;
+      if (!own) p = -1;
+    }
+  }
+  int4 e[kPre];
+#pragma unroll
+  for (int t = 0; t < kPre; ++t)
+    e[t] = (l + t * g < ng) ? ld_stream_v4(row + l + t * g) : make_int4(-1, -1, -1, -1);
+
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  uint64_t keep;
+  asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
+  const int cur = A.cur;
+  const Gsrc G{A.y[cur], A.yh[cur], keep, (uint32_t)A.M};
+  float2 ym = make_float2(0.f, 0.f), v = ym, s2 = ym;
+  if (p >= 0) ym = G.y[p];
+  const float2 yi = f32_pos<POS>() ? ym : (p >= 0 ? load_pos<POS>(G.y, G.yh, (uint32_t)p) : ym);
+  if (own) {
+    v = A.v[0][p];
+    if (MODE == kAdadelta) s2 = A.s2[p];
+  }
+  float fx = 0.f, fy = 0.f;
+  if (l < ng) {
+    if (l + g < ng) {
+      visit8<MODE, POS, METRIC>(e[0], e[1], G, yi, A.c, fx, fy);
+      if (l + 3 * g < ng)
+        visit8<MODE, POS, METRIC>(e[2], e[3], G, yi, A.c, fx, fy);
+      else if (l + 2 * g < ng)
+        visit4<MODE, POS, METRIC>(e[2], G, yi, A.c, fx, fy);
+    } else {
+      visit4<MODE, POS, METRIC>(e[0], G, yi, A.c, fx, fy);
+    }
+  }
+  int at = l + kPre * g;
+  for (; at + g < ng; at += 2 * g) {
+    const int4 ea = ld_stream_v4(row + at);
+    const int4 eb = ld_stream_v4(row + at + g);
+    visit8<MODE, POS, METRIC>(ea, eb, G, yi, A.c, fx, fy);
+  }
+  if (at < ng) visit4<MODE, POS, METRIC>(ld_stream_v4(row + at), G, yi, A.c, fx, fy);
+  if (wide) {
+    __shared__ float wred[2][kMaxStepBlock / 32];
+    group_sum(fx, fy, 32);
+    if (lane == 0) {
+      wred[0][wib] = fx;
+      wred[1][wib] = fy;
+    }
+    __syncthreads();
+    if (own) {
+      const int w0 = grp * kWideWarps;
+      fx = wred[0][w0];
+      fy = wred[1][w0];
+      for (int q = 1; q < kWideWarps; ++q) {
+        fx += wred[0][w0 + q];
+        fy += wred[1][w0 + q];
+      }
+    }
+  } else if (hub) {
+    group_sum(fx, fy, g);
+  }
+  if (!own) return;
+  float2 yn;
+  if (MODE == kMomentum) {
+    float2 vn;
+    momentum_update(A.a, A.b, fx, fy, ym, v, vn, yn);
+    v = vn;
+  } else if (MODE == kNesterov) {
+    float2 vn;
+    nesterov_update(A.a, A.b, fx, fy, ym, v, vn, yn);
+    v = vn;
+  } else {
+    adadelta_update(A.rho, A.eps, fx, fy, ym, v, s2, yn);
+    A.s2[p] = s2;
+  }
+  A.v[0][p] = v;
+  A.y[cur ^ 1][p] = yn;
+  if constexpr (!f32_pos<POS>()) A.yh[cur ^ 1][p] = round_pos<POS>(yn);
+}
+
 // ---- persistent grid kernel ------------------------------------------------------
 //
 // All steps of an ivhd_step call in one cooperative launch: every block is
@@ -1501,8 +1635,15 @@ int step_grid(const ivhd_ctx* ctx) {
   return (int)(nb_wide + nb_hub + nb_sell);
 }
 
+// Grids up to this many blocks of 128 threads take k_step_ahead: about half of
+// what the GPU holds, so that the next grid fits beside it.  Measured, us per
+// step with k_step / k_step_ahead: 94 blocks 3.04 / 2.63, 314 3.56 / 3.27, 358
+// 4.36 / 3.74, 639 4.52 / 4.01, 754 4.42 / 4.40, 1,730 5.79 / 7.35.
+constexpr int kAheadBlocks = 704;
+// first: the launch follows the layout's own kernels, whose writes a dependent
+// launch could not count on before its wait.
 template <int MODE, int POS, int METRIC, bool ADAPT>
-static void launch1(int grid, cudaStream_t s, const StepArgs& A) {
+static void launch1(int grid, cudaStream_t s, const StepArgs& A, bool first) {
   // programmatic dependent launch: the next step's blocks start while this
   // step's last wave drains (0.5 % at 1.4e6 vertices, 5 % at 2,000)
   cudaLaunchConfig_t cfg = {};
@@ -1514,36 +1655,43 @@ static void launch1(int grid, cudaStream_t s, const StepArgs& A) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = first ? 0 : 1;
+  if constexpr (!ADAPT) {
+    if (grid * (A.wpb / 4) <= kAheadBlocks) {
+      cudaLaunchKernelEx(&cfg, k_step_ahead<MODE, POS, METRIC>, A);
+      return;
+    }
+  }
   cudaLaunchKernelEx(&cfg, k_step<MODE, POS, METRIC, ADAPT>, A);
 }
 
 template <int POS, int METRIC>
-static void launch_opt(int opt, bool adapt, int grid, cudaStream_t s, const StepArgs& A) {
+static void launch_opt(int opt, bool adapt, int grid, cudaStream_t s, const StepArgs& A,
+                       bool first) {
   switch (opt) {
     case IVHD_OPT_NESTEROV:
       if (adapt)
-        launch1<kNesterov, POS, METRIC, true>(grid, s, A);
+        launch1<kNesterov, POS, METRIC, true>(grid, s, A, first);
       else
-        launch1<kNesterov, POS, METRIC, false>(grid, s, A);
+        launch1<kNesterov, POS, METRIC, false>(grid, s, A, first);
       break;
-    case IVHD_OPT_ADADELTA: launch1<kAdadelta, POS, METRIC, false>(grid, s, A); break;
+    case IVHD_OPT_ADADELTA: launch1<kAdadelta, POS, METRIC, false>(grid, s, A, first); break;
     default:
       if (adapt)
-        launch1<kMomentum, POS, METRIC, true>(grid, s, A);
+        launch1<kMomentum, POS, METRIC, true>(grid, s, A, first);
       else
-        launch1<kMomentum, POS, METRIC, false>(grid, s, A);
+        launch1<kMomentum, POS, METRIC, false>(grid, s, A, first);
       break;
   }
 }
 
 template <int METRIC>
 static void launch_pos(const ivhd_ctx* ctx, bool adapt, int grid, cudaStream_t s,
-                       const StepArgs& A) {
+                       const StepArgs& A, bool first) {
   switch (ctx->p.pos_format) {
-    case IVHD_POS_F16: launch_opt<IVHD_POS_F16, METRIC>(ctx->p.opt, adapt, grid, s, A); break;
-    case IVHD_POS_BF16: launch_opt<IVHD_POS_BF16, METRIC>(ctx->p.opt, adapt, grid, s, A); break;
-    default: launch_opt<IVHD_POS_F32, METRIC>(ctx->p.opt, adapt, grid, s, A); break;
+    case IVHD_POS_F16: launch_opt<IVHD_POS_F16, METRIC>(ctx->p.opt, adapt, grid, s, A, first); break;
+    case IVHD_POS_BF16: launch_opt<IVHD_POS_BF16, METRIC>(ctx->p.opt, adapt, grid, s, A, first); break;
+    default: launch_opt<IVHD_POS_F32, METRIC>(ctx->p.opt, adapt, grid, s, A, first); break;
   }
 }
 
@@ -1552,10 +1700,13 @@ cudaError_t launch_step(ivhd_ctx* ctx, int cur, cudaStream_t s) {
   const StepArgs A = make_args(ctx, cur);
   const int grid = step_grid(ctx);
   const bool adapt = ctx->p.adaptive != 0;
+  // a captured step starts behind whatever the graph is launched behind
+  const bool first = ctx->layout_fresh && s == ctx->stream;
+  if (first) ctx->layout_fresh = false;
   if (ctx->metric == IVHD_METRIC_L1)
-    launch_pos<IVHD_METRIC_L1>(ctx, adapt, grid, s, A);
+    launch_pos<IVHD_METRIC_L1>(ctx, adapt, grid, s, A, first);
   else
-    launch_pos<IVHD_METRIC_L2>(ctx, adapt, grid, s, A);
+    launch_pos<IVHD_METRIC_L2>(ctx, adapt, grid, s, A, first);
   if (adapt) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1);
