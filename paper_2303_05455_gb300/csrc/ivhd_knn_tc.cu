@@ -29,17 +29,23 @@
 // (the nearest-neighbour placement of Progressive UMAP, Sec. 2.4.3); the
 // arithmetic and the certificate are the same, with n_i the query's norm.
 //
-// One CTA owns 128 query rows (the 128 tensor-memory lanes) and sweeps all
-// candidates in tiles of 256 columns:
-//   warp 0, one lane   TMA producer: 128 x 64 query and 256 x 64 candidate
-//                      slices into a 4-stage ring (128-byte swizzle)
-//   warp 1, one lane   MMA issuer: tcgen05.mma M=128 N=256 K=16 into one of two
-//                      256-column accumulators in tensor memory (512 columns),
-//                      so the epilogue of tile t overlaps the MMAs of tile t+1
-//   warps 2-5          epilogue: thread = query row; tcgen05.ld of 32 columns at
-//                      a time, distance, compare with the row's list held in
-//                      registers
+// A pair of CTAs (a cluster of two, cta_group::2) owns 256 query rows, 128
+// tensor-memory lanes each, and sweeps all candidates in tiles of 256 columns:
+//   warp 0, one lane   TMA producer: this CTA's 128 x 64 query slice and its
+//                      half (128 x 64) of the candidate slice into a 6-stage
+//                      ring (128-byte swizzle); 32 KB from L2 per 512 clocks of
+//                      MMAs instead of 48 KB with a tile per CTA
+//   warp 1, one lane   (rank 0) MMA issuer: tcgen05.mma M=256 N=256 K=16 into one
+//                      of two 256-column accumulators in tensor memory, so the
+//                      epilogue of tile t overlaps the MMAs of tile t+1
+//   warps 2-9          epilogue: thread = query row; tcgen05.ld of 16 columns at
+//                      a time, distance, test against the row's threshold, a
+//                      queue in shared memory and a list in registers
 // Every wait is bounded; a timeout sets an error flag and all roles stop.
+// What bounds it (kernel alone, M = 100,000 floats x 100, K = 320): 3.6 ms with
+// the epilogue doing nothing (1.77 PFLOP/s, the tensor cores at their power
+// limit), 3.7 ms with its tests but no candidate passing; handling the
+// candidates takes the rest.
 #include <climits>
 #include <cstdint>
 #include <cstring>
@@ -54,18 +60,19 @@ namespace {
 
 using namespace tc;
 
-constexpr int kTM = 128;  // query rows per CTA
-constexpr int kTN = 256;  // candidate columns per accumulator tile
-constexpr int kTStages = 4;
+constexpr int kTM = 128;  // query rows per CTA (two CTAs share a 256-row tile)
+constexpr int kTN = 256;  // candidate columns per accumulator tile, half of them loaded by each CTA
+constexpr int kTStages = 6;
 constexpr int kEpiWarps = 8;  // two warpgroups: each reads one 128-column half of a tile
 constexpr int kTcThreads = 32 * (2 + kEpiWarps);
 constexpr int kMaxKnnSegments = 32;  // column segments of one kNN launch (short query sets)
 constexpr int kGroup = 8;            // columns tested and queued together in the epilogue
+constexpr int kChunk = 16;           // columns read from tensor memory at once
 constexpr int kQueue = 14;           // candidates a row holds back before its list takes them
 
 struct KnnSmem {
   static constexpr int a_bytes = kTM * kBK * 2;
-  static constexpr int b_bytes = kTN * kBK * 2;
+  static constexpr int b_bytes = kTN / 2 * kBK * 2;
   static constexpr int stage_bytes = a_bytes + b_bytes;
   static constexpr int bar_offset = kTStages * stage_bytes;
   static constexpr int nrm_offset = bar_offset + 256;  // 8 warps x 128 column terms
@@ -96,15 +103,24 @@ __device__ __forceinline__ void list_insert(D d, int j, D (&dl)[L], int (&jl)[L]
   }
 }
 
-// Bounded wait that also stops when another role has given up.
+// Bounded wait that also stops when another role of either CTA has given up.
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity,
                                               volatile int* abort_flag) {
   for (uint32_t it = 0; it < kSpinLimit; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 255u) == 255u && *abort_flag) return false;
   }
-  *abort_flag = 1;
+  for (uint32_t r = 0; r < 2; ++r) st_cluster_u32(pair_addr((const void*)abort_flag, r), 1u);
   return false;
+}
+
+// Floats as integers of the same order, and back.
+__device__ __forceinline__ int ordered_int(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float ordered_float(int i) {
+  return __int_as_float(i ^ ((i >> 31) & 0x7fffffff));
 }
 
 // Twice the certificate's bound over a row's distances: a vertex whose key is
@@ -121,7 +137,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
              const float* __restrict__ nrm_f, const int32_t* __restrict__ nrm_i,
              const float* __restrict__ qnrm_f, const int32_t* __restrict__ qnrm_i, int Mq, int M,
              int Kp, bool self, int k, int seg_tiles, float eps_coef,
-             int32_t* __restrict__ out_ids, float* __restrict__ out_d, int32_t* __restrict__ err) {
+             int32_t* __restrict__ bounds, int32_t* __restrict__ out_ids,
+             float* __restrict__ out_d, int32_t* __restrict__ err) {
   using D = typename std::conditional<U8, int32_t, float>::type;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -132,10 +149,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint64_t* done = acc_empty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* issued = abort_flag + 1;
   constexpr uint32_t kCols = 2 * kTN;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cta_rank();  // 0: the CTA that issues the MMAs of the pair
   const int m0 = blockIdx.x * kTM;
   const int nk = Kp / kBK;
   // this CTA's column segment: tiles t0 .. t0 + n_tiles - 1 (blockIdx.y of gridDim.y)
@@ -150,30 +167,32 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 32 * kEpiWarps);  // every epilogue thread arrives
+      mbar_init(&acc_empty[b], 2 * kEpiWarps);  // every epilogue warp of both CTAs arrives
     }
     mbar_init(done, 1);
     *abort_flag = 0;
-    *issued = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(kCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
+  pair_sync();  // both CTAs' barriers are set up before either signals the other's
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
     if (lane == 0) {
-      // producer: the query slice (re-read from L2 for every tile) and the candidate slice
+      // producer: this CTA's query slice (re-read from L2 for every tile) and
+      // its half of the candidate slice; the bytes of both CTAs are counted by
+      // the barrier of rank 0
       uint32_t g = 0;
-      for (int t = 0; t < n_tiles; ++t) {
-        bool ok = true;
+      bool ok = true;
+      for (int t = 0; t < n_tiles && ok; ++t) {
         for (int kt = 0; kt < nk; ++kt, ++g) {
           const int s = (int)(g % kTStages);
           if (g >= kTStages && !wait_or_abort(&empty[s], ((g / kTStages) - 1) & 1, abort_flag)) {
@@ -183,17 +202,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           }
           unsigned char* sa = smem + s * KnnSmem::stage_bytes;
           unsigned char* sb = sa + KnnSmem::a_bytes;
-          mbar_expect_tx(&full[s], KnnSmem::stage_bytes);
-          tma_load_2d(sa, &map_a, kt * kBK, m0, &full[s]);
-          tma_load_2d(sb, &map_b, kt * kBK, (t0 + t) * kTN, &full[s]);
-          *issued = (int)(g + 1);
+          if (rank == 0) mbar_expect_tx(&full[s], 2 * KnnSmem::stage_bytes);
+          const uint32_t bar = pair_addr(&full[s], 0);
+          tma_load_2d_pair(sa, &map_a, kt * kBK, m0, bar);
+          tma_load_2d_pair(sb, &map_b, kt * kBK, (t0 + t) * kTN + (int)rank * (kTN / 2), bar);
         }
-        if (!ok) break;
       }
+      // a copy in flight lands within microseconds: after an abort, time for
+      // it before the shared memory goes away
+      if (!ok)
+        for (int it = 0; it < 2000; ++it) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc_bf16(kTM, kTN);
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = instr_desc_bf16(2 * kTM, kTN);
       uint32_t g = 0;
       bool ok = true;
       for (int t = 0; t < n_tiles && ok; ++t) {
@@ -216,14 +238,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           const uint32_t sb = sa + KnnSmem::a_bytes;
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk)
-            umma_bf16(dst, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32), idesc,
-                      (kt > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(&empty[s]);
+            umma_bf16_pair(dst, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32),
+                           idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+          umma_commit_pair(&empty[s]);
         }
-        if (ok) umma_commit(&acc_full[b]);
+        if (ok) umma_commit_pair(&acc_full[b]);
       }
       // every MMA issued above has finished before tensor memory is released
-      umma_commit(done);
+      // and either CTA's shared memory goes away
+      umma_commit_pair(done);
       if (!mbar_wait(done, 0)) atomicOr(err, 8);
     }
   } else {
@@ -239,7 +262,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // candidate, whatever the other rows do) and goes to the lists when some row
     // of the warp has a full queue, all rows together: inserting each candidate
     // at once made the whole warp walk one row's list, and that, not the tensor
-    // cores, set the time (whole build, 300,000 x 100 floats, k = 5: 70.4 -> 44.2 ms).
+    // cores, set the time (whole build, 300,000 x 100 floats, k = 5: 70.4 -> 44.2 ms
+    // with queues, 42.7 with appends that do not branch, loads that run ahead and
+    // shared bounds; 70,000 x 784 bytes 6.00 -> 5.59 -> 5.01 ms).
     // uint8: the float key and the float threshold are within 2 of the exact
     // integers (magnitudes below 2^26), so the test allows 16 and the queue takes
     // the exact keys.
@@ -250,13 +275,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int i = m0 + r;
     // the half-tile's 128 column terms, staged per warp; each lane prefetches
     // its 4 terms of the next tile into registers while the current one is processed
-    float* nbuf = reinterpret_cast<float*>(smem + KnnSmem::nrm_offset) + (warp - 2) * kHalf;
+    const uint32_t nbuf = smem_u32(smem + KnnSmem::nrm_offset) + (uint32_t)(warp - 2) * kHalf * 4;
     constexpr int kPer = kHalf / 32;
-    constexpr int kQueueStride = 32 * kEpiWarps;
-    int2* const queue = reinterpret_cast<int2*>(smem + KnnSmem::queue_offset) + (warp - 2) * 32 + lane;
+    constexpr int kQueueStride = 32 * kEpiWarps * 8;  // bytes from one entry of a row to the next
+    const uint32_t queue = smem_u32(smem + KnnSmem::queue_offset) + ((warp - 2) * 32 + lane) * 8;
     const D kMaxKey = U8 ? (D)INT_MAX : (D)__int_as_float(0x7f800000);
     const float kInf = __int_as_float(0x7f800000);
     const float col_scale = 1.f - eps_coef;
+    const bool has_row = i < Mq;
+    int shared_bound = INT_MAX;  // bounds[i] as of the last fetch
     float pn[kPer];
     auto fetch = [&](int t) {
 #pragma unroll
@@ -267,6 +294,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         else
           pn[e] = (jc < M) ? col_scale * nrm_f[jc] : 0.f;
       }
+      if (has_row) shared_bound = *reinterpret_cast<volatile int32_t*>(bounds + i);
     };
     D dl[L];
     int jl[L];
@@ -281,32 +309,89 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // key (uint8) or, float, the k-th key plus what separates its distance's
     // upper bound from a lower bound: slack = 2 eps (n_i + max n_j).
     const float slack = U8 ? 0.f : key_slack(eps_coef, (float)ni, nrm_f[M]);
+    // The row's lists (the other half's, and those of the other column segments)
+    // share the smallest of their bounds: together they let pass about as much
+    // as one list would, and a segment that starts late starts with a bound.
+    // (uint8: a key equal to another list's k-th may have the lower index, so
+    // only larger ones are dropped.)
     D thr = kMaxKey;
     float thr_f = kInf;
-    int held = 0;
+    auto tighten = [&](D t) {
+      thr = min(thr, t);
+      thr_f = U8 ? (thr == (D)INT_MAX ? kInf : (float)thr + 16.f) : (float)thr;
+    };
+    uint32_t qa = queue;         // end of the row's queue
     auto flush = [&]() {
+      const int held = (int)(qa - queue) / kQueueStride;
       const int most = __reduce_max_sync(0xffffffffu, held);
       for (int q = 0; q < most; ++q) {
         D d = kMaxKey;
         int j = INT_MAX;
         if (q < held) {
-          const int2 e = queue[q * kQueueStride];
+          const int2 e = ld_shared_i2(queue + q * kQueueStride);
           d = U8 ? (D)e.x : (D)__int_as_float(e.x);
           j = e.y;
         }
         list_insert<D, L>(d, j, dl, jl);
       }
-      held = 0;
+      qa = queue;
       D dk = dl[L - 1];  // the k-th key: the smallest from there on
 #pragma unroll
       for (int q = 0; q < L; ++q)
         if (q >= k - 1) dk = min(dk, dl[q]);
       if constexpr (U8) {
-        thr = dk;
-        thr_f = dk == INT_MAX ? kInf : (float)dk + 16.f;
+        if (has_row && dk != INT_MAX) atomicMin(bounds + i, dk + 1);
+        tighten(dk);
       } else {
-        thr = fminf(dl[L - 1], dk + slack);
-        thr_f = thr;
+        if (has_row && dk < kInf) atomicMin(bounds + i, ordered_int(dk + slack));
+        tighten(fminf(dl[L - 1], dk + slack));
+      }
+    };
+    // kChunk columns from c0 of this half tile, which starts at column n0
+    auto process = [&](const uint32_t(&v)[kChunk], int n0, int c0) {
+      const int jb = n0 + c0;
+      if (jb >= M) return;
+      float d[kChunk];
+#pragma unroll
+      for (int q = 0; q < kChunk; q += 4) {
+        const float4 w = ld_shared_f4(nbuf + (c0 + q) * 4);
+        d[q + 0] = fmaf(-2.f, __uint_as_float(v[q + 0]), w.x);
+        d[q + 1] = fmaf(-2.f, __uint_as_float(v[q + 1]), w.y);
+        d[q + 2] = fmaf(-2.f, __uint_as_float(v[q + 2]), w.z);
+        d[q + 3] = fmaf(-2.f, __uint_as_float(v[q + 3]), w.w);
+      }
+      if (jb + kChunk - 1 >= M || (jb <= iself && iself <= jb + kChunk - 1)) {
+#pragma unroll
+        for (int q = 0; q < kChunk; ++q)
+          if (jb + q >= M || jb + q == iself) d[q] = kInf;
+      }
+      unsigned any[kChunk / kGroup];
+#pragma unroll
+      for (int g = 0; g < kChunk; g += kGroup) {
+        const float a = fminf(fminf(d[g], d[g + 1]), fminf(d[g + 2], d[g + 3]));
+        const float b = fminf(fminf(d[g + 4], d[g + 5]), fminf(d[g + 6], d[g + 7]));
+        any[g / kGroup] = __ballot_sync(0xffffffffu, fminf(a, b) < thr_f);
+      }
+#pragma unroll
+      for (int g = 0; g < kChunk; g += kGroup) {
+        if (any[g / kGroup] == 0) continue;
+        if constexpr (U8) {
+#pragma unroll
+          for (int q = 0; q < kGroup; q += 4) {
+            const float4 w = ld_shared_f4(nbuf + (c0 + g + q) * 4);
+            const float nj[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int key = (int)nj[u] - 2 * __float2int_rn(__uint_as_float(v[g + q + u]));
+              append_shared<kQueueStride>(qa, d[g + q + u] < thr_f && key < thr, key, jb + g + q + u);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < kGroup; ++q)
+            append_shared<kQueueStride>(qa, d[g + q] < thr_f, __float_as_int(d[g + q]), jb + g + q);
+        }
+        if (__any_sync(0xffffffffu, qa > queue + (kQueue - kGroup) * kQueueStride)) flush();
       }
     };
     bool ok = true;
@@ -321,51 +406,27 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       asm volatile("tcgen05.fence::after_thread_sync;");
       __syncwarp();
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) nbuf[e * 32 + lane] = pn[e];
+      for (int e = 0; e < kPer; ++e) st_shared_f32(nbuf + (e * 32 + lane) * 4, pn[e]);
       __syncwarp();
+      tighten(U8 ? (D)shared_bound : (D)ordered_float(shared_bound));
       if (t + 1 < n_tiles) fetch(t + 1);
       const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * kTN + half * kHalf);
       const int n0 = (t0 + t) * kTN + half * kHalf;
-      for (int c0 = 0; c0 < kHalf && n0 + c0 < M; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld32(tbase + c0, v);
-        const int jb = n0 + c0;
-        float d[32];
-#pragma unroll
-        for (int q = 0; q < 32; q += 4) {
-          const float4 w = *reinterpret_cast<const float4*>(nbuf + c0 + q);
-          d[q + 0] = fmaf(-2.f, __uint_as_float(v[q + 0]), w.x);
-          d[q + 1] = fmaf(-2.f, __uint_as_float(v[q + 1]), w.y);
-          d[q + 2] = fmaf(-2.f, __uint_as_float(v[q + 2]), w.z);
-          d[q + 3] = fmaf(-2.f, __uint_as_float(v[q + 3]), w.w);
-        }
-        if (jb + 31 >= M || (jb <= iself && iself <= jb + 31)) {
-#pragma unroll
-          for (int q = 0; q < 32; ++q)
-            if (jb + q >= M || jb + q == iself) d[q] = kInf;
-        }
-#pragma unroll
-        for (int g = 0; g < 32; g += kGroup) {
-          float mn = d[g];
-#pragma unroll
-          for (int q = 1; q < kGroup; ++q) mn = fminf(mn, d[g + q]);
-          if (!__any_sync(0xffffffffu, mn < thr_f)) continue;
-#pragma unroll
-          for (int q = 0; q < kGroup; ++q) {
-            if (d[g + q] < thr_f) {
-              if constexpr (U8) {
-                const int e = (int)nbuf[c0 + g + q] - 2 * __float2int_rn(__uint_as_float(v[g + q]));
-                if (e < thr) queue[held++ * kQueueStride] = make_int2(e, jb + g + q);
-              } else {
-                queue[held++ * kQueueStride] = make_int2(__float_as_int(d[g + q]), jb + g + q);
-              }
-            }
-          }
-          if (__any_sync(0xffffffffu, held > kQueue - kGroup)) flush();
-        }
+      // the load of the next columns runs while the current ones are tested
+      uint32_t va[kChunk], vb[kChunk];
+      tmem_ld16_nowait(tbase, va);
+#pragma unroll 1
+      for (int c0 = 0; c0 < kHalf; c0 += 2 * kChunk) {
+        tmem_wait_ld16(va);
+        tmem_ld16_nowait(tbase + c0 + kChunk, vb);
+        process(va, n0, c0);
+        tmem_wait_ld16(vb);
+        if (c0 + 2 * kChunk < kHalf) tmem_ld16_nowait(tbase + c0 + 2 * kChunk, va);
+        process(vb, n0, c0 + kChunk);
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
-      mbar_arrive(&acc_empty[b]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(pair_addr(&acc_empty[b], 0));
     }
     if (ok) flush();
     if (ok && i < Mq) {
@@ -384,17 +445,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     if (!ok && lane == 0) atomicOr(err, 16);
   }
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) {
-    // drain copies still in flight before the shared memory goes away
-    const int iss = *issued;
-    for (int g = (iss > kTStages ? iss - kTStages : 0); g < iss; ++g)
-      mbar_wait(&full[g % kTStages], (g / kTStages) & 1);
-  }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
+  pair_sync();  // no MMA, copy or arrival of the pair is outstanding
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
 // ---- operand preparation ---------------------------------------------------
@@ -660,7 +715,11 @@ template <bool U8, int L>
 cudaError_t launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, const float* nrm_f,
                       const int32_t* nrm_i, const float* qnrm_f, const int32_t* qnrm_i, int Mq,
                       int M, int Kp, bool self, int k, int segments, int seg_tiles, float eps_coef,
-                      int32_t* out_ids, float* out_d, int32_t* err, cudaStream_t s) {
+                      int32_t* bounds, int32_t* out_ids, float* out_d, int32_t* err,
+                      cudaStream_t s) {
+  // no bound yet: larger than any key, and as a float 3.4e38
+  const cudaError_t e0 = cudaMemsetAsync(bounds, 0x7f, (size_t)Mq * sizeof(int32_t), s);
+  if (e0 != cudaSuccess) return e0;
   static bool attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -671,11 +730,20 @@ cudaError_t launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, const float*
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
-  const dim3 grid((unsigned)((Mq + kTM - 1) / kTM), (unsigned)segments);
-  k_knn_tc<U8, L><<<grid, kTcThreads, KnnSmem::total, s>>>(
-      ma, mb, nrm_f, nrm_i, qnrm_f, qnrm_i, Mq, M, Kp, self, k, seg_tiles, eps_coef, out_ids,
-      out_d, err);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * (unsigned)((Mq + 2 * kTM - 1) / (2 * kTM)), (unsigned)segments);
+  cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = KnnSmem::total;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_knn_tc<U8, L>, ma, mb, nrm_f, nrm_i, qnrm_f, qnrm_i, Mq, M, Kp,
+                            self, k, seg_tiles, eps_coef, bounds, out_ids, out_d, err);
 }
 
 }  // namespace
@@ -752,13 +820,14 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
   __nv_bfloat16* B = base ? const_cast<__nv_bfloat16*>(base->B) : b.get<__nv_bfloat16>(M * Kp);
   __nv_bfloat16* A = (u8 && P.self) ? B : b.get<__nv_bfloat16>(Mq * Kp);
   int32_t* err = b.get<int32_t>(8);  // err, n_fb, max-err bits
+  int32_t* bounds = b.get<int32_t>(Mq);
   if (!b.ok) return IVHD_ERR_OOM;
   cudaError_t e = cudaMemsetAsync(err, 0, 8 * sizeof(int32_t), s);
   int32_t* n_fb = err + 1;
   int32_t* maxerr_bits = err + 2;
   auto blocks = [](int64_t n) { return (unsigned)((n + 255) / 256); };
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A, Mq, Kp, Kp, kTM) || !make_map(&mb, B, M, Kp, Kp, kTN))
+  if (!make_map(&ma, A, Mq, Kp, Kp, kTM) || !make_map(&mb, B, M, Kp, Kp, kTN / 2))
     return IVHD_ERR_CUDA;
   const float eps_coef = (float)(1.0 / 8192.0 + (double)N / 524288.0);
   // Short query sets: the columns are split into segments (one CTA per row
@@ -770,7 +839,7 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return IVHD_ERR_CUDA;
-  const int64_t row_blocks = (Mq + kTM - 1) / kTM;
+  const int64_t row_blocks = 2 * ((Mq + 2 * kTM - 1) / (2 * kTM));
   const int all_tiles = (int)((M + kTN - 1) / kTN);
   int want = 1;
   int64_t best_cost = INT64_MAX;
@@ -804,10 +873,10 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
         k_norms_u8s<<<blocks(Mq), 256, 0, s>>>(Q, Mq, N, qnrm);
       }
       e = (L == 8) ? launch_tc<true, 8>(ma, mb, nullptr, nrm, nullptr, qnrm, (int)Mq, (int)M, Kp,
-                                        P.self, k, segs, seg_tiles, 0.f, lids, (float*)lkeys, err,
+                                        P.self, k, segs, seg_tiles, 0.f, bounds, lids, (float*)lkeys, err,
                                         s)
                    : launch_tc<true, kKnnList>(ma, mb, nullptr, nrm, nullptr, qnrm, (int)Mq,
-                                               (int)M, Kp, P.self, k, segs, seg_tiles, 0.f, lids,
+                                               (int)M, Kp, P.self, k, segs, seg_tiles, 0.f, bounds, lids,
                                                (float*)lkeys, err, s);
     }
     if (e == cudaSuccess) {
@@ -839,10 +908,10 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
     }
     if (e == cudaSuccess) {
       e = (L == 16) ? launch_tc<false, 16>(ma, mb, nrm, nullptr, qnrm, nullptr, (int)Mq, (int)M,
-                                           Kp, P.self, k, segs, seg_tiles, eps_coef, cand, cd, err, s)
+                                           Kp, P.self, k, segs, seg_tiles, eps_coef, bounds, cand, cd, err, s)
                     : launch_tc<false, kKnnList>(ma, mb, nrm, nullptr, qnrm, nullptr, (int)Mq,
                                                  (int)M, Kp, P.self, k, segs, seg_tiles, eps_coef,
-                                                 cand, cd, err, s);
+                                                 bounds, cand, cd, err, s);
     }
     if (e == cudaSuccess) {
       const unsigned g8 = (unsigned)((Mq + 7) / 8);
