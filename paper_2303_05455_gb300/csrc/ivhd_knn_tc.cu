@@ -103,17 +103,6 @@ __device__ __forceinline__ void list_insert(D d, int j, D (&dl)[L], int (&jl)[L]
   }
 }
 
-// Bounded wait that also stops when another role of either CTA has given up.
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity,
-                                              volatile int* abort_flag) {
-  for (uint32_t it = 0; it < kSpinLimit; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 255u && *abort_flag) return false;
-  }
-  for (uint32_t r = 0; r < 2; ++r) st_cluster_u32(pair_addr((const void*)abort_flag, r), 1u);
-  return false;
-}
-
 // Floats as integers of the same order, and back.
 __device__ __forceinline__ int ordered_int(float f) {
   const int i = __float_as_int(f);
@@ -195,7 +184,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       for (int t = 0; t < n_tiles && ok; ++t) {
         for (int kt = 0; kt < nk; ++kt, ++g) {
           const int s = (int)(g % kTStages);
-          if (g >= kTStages && !wait_or_abort(&empty[s], ((g / kTStages) - 1) & 1, abort_flag)) {
+          if (g >= kTStages && !pair_wait(&empty[s], ((g / kTStages) - 1) & 1, abort_flag)) {
             atomicOr(err, 1);
             ok = false;
             break;
@@ -220,7 +209,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       bool ok = true;
       for (int t = 0; t < n_tiles && ok; ++t) {
         const int b = t & 1;
-        if (t >= 2 && !wait_or_abort(&acc_empty[b], ((t >> 1) - 1) & 1, abort_flag)) {
+        if (t >= 2 && !pair_wait(&acc_empty[b], ((t >> 1) - 1) & 1, abort_flag)) {
           atomicOr(err, 2);
           break;
         }
@@ -228,7 +217,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const uint32_t dst = tmem + (uint32_t)(b * kTN);
         for (int kt = 0; kt < nk; ++kt, ++g) {
           const int s = (int)(g % kTStages);
-          if (!wait_or_abort(&full[s], (g / kTStages) & 1, abort_flag)) {
+          if (!pair_wait(&full[s], (g / kTStages) & 1, abort_flag)) {
             atomicOr(err, 4);
             ok = false;
             break;
@@ -398,7 +387,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     fetch(0);
     for (int t = 0; t < n_tiles; ++t) {
       const int b = t & 1;
-      if (!wait_or_abort(&acc_full[b], (t >> 1) & 1, abort_flag)) ok = false;
+      if (!pair_wait(&acc_full[b], (t >> 1) & 1, abort_flag)) ok = false;
       if (!__all_sync(0xffffffffu, ok)) {  // the warp stays together below
         ok = false;
         break;

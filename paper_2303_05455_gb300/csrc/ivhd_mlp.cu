@@ -20,6 +20,7 @@
 
 #include "ivhd_gemm.cuh"
 #include "ivhd_internal.cuh"
+#include "ivhd_mlp_place.cuh"
 
 struct ivhd_mlp {
   int n_in = 0, hidden = 0, max_batch = 0;
@@ -27,6 +28,7 @@ struct ivhd_mlp {
   int64_t n_params = 0;
   int64_t t = 0;          // Adam step counter
   int last_rows = 0;      // rows of the last batch whose intermediates are held
+  bool pending = false;   // that batch went through the one-kernel path: h1 and h2 are not held yet
   bool poisoned = false;
   // parameters: FP32 master, Adam moments, gradients (flat: W1 b1 W2 b2 W3 b3)
   float* w = nullptr;
@@ -511,11 +513,80 @@ cudaError_t loss_grad(ivhd_mlp* P, const float* tgt, int B, bool sum_weights = t
   return e;
 }
 
-cudaError_t load_x(ivhd_mlp* P, const void* x, int dtype, float scale, int64_t rows) {
+cudaError_t convert_x(ivhd_mlp* P, const void* x, int dtype, float scale, int64_t rows,
+                      __nv_bfloat16* out, cudaStream_t s) {
   const int64_t n = rows * P->n_in;
-  k_convert_x<<<nb((n + 7) / 8), 256, 0, P->stream>>>(x, dtype, scale, n, P->xb);
+  k_convert_x<<<nb((n + 7) / 8), 256, 0, s>>>(x, dtype, scale, n, out);
   ++P->launches;
   return cudaGetLastError();
+}
+
+cudaError_t load_x(ivhd_mlp* P, const void* x, int dtype, float scale, int64_t rows) {
+  P->pending = false;
+  return convert_x(P, x, dtype, scale, rows, P->xb, P->stream);
+}
+
+// The intermediates of a batch that went through the one-kernel path, from its
+// input rows (still in P->xb) and the weights it used.
+cudaError_t hold_activations(ivhd_mlp* P) {
+  if (!P->pending) return cudaSuccess;
+  P->pending = false;
+  return forward(P, P->last_rows);
+}
+
+// n rows through the one-kernel path.  The last chunk is that of the
+// layer-by-layer path (the rows after the last multiple of max_batch below n):
+// its input ends in P->xb and its outputs also in P->y, where
+// ivhd_mlp_activations looks for them.  The rows before it go in chunks of
+// whole rounds of tiles.  The next chunk is converted on the side stream, into
+// the buffer that the training step uses for the transposed input, while the
+// current one runs.
+cudaError_t place(ivhd_mlp* P, const void* x, int dtype, float scale, int64_t n, float* y) {
+  const Offs o = offsets(P->n_in, P->hidden);
+  const MlpPlace net{P->n_in,      P->hidden,   P->w1,        P->w2,        P->w + o.b1,
+                     P->w + o.b2,  P->w + o.W3, P->w + o.b3,  P->err};
+  const size_t esz = dtype == 1 ? 1 : (dtype == 2 ? 4 : 2);
+  const int64_t last0 = (n - 1) / P->max_batch * P->max_batch;
+  const int64_t B = mlp_place_rows(P->max_batch), chunks = (last0 + B - 1) / B + 1;
+  cudaStream_t s = P->stream, side = P->side;
+  // events: [0], [1] converted (even, odd chunk), [2], [3] consumed, [4] start
+  auto buf = [&](int64_t i) { return ((chunks - 1 - i) & 1) ? P->xt : P->xb; };
+  auto first = [&](int64_t i) { return i + 1 < chunks ? i * B : last0; };
+  auto rows_of = [&](int64_t i) {
+    return i + 1 < chunks ? (last0 - i * B < B ? last0 - i * B : B) : n - last0;
+  };
+  cudaError_t e = cudaSuccess;
+  auto chk = [&](cudaError_t v) {
+    if (e == cudaSuccess) e = v;
+  };
+  auto convert = [&](int64_t i, cudaStream_t st) {
+    chk(convert_x(P, (const char*)x + (size_t)first(i) * P->n_in * esz, dtype, scale, rows_of(i),
+                  buf(i), st));
+  };
+  P->pending = false;
+  convert(0, s);
+  if (chunks > 1) {
+    chk(cudaEventRecord(P->ev[4], s));
+    chk(cudaStreamWaitEvent(side, P->ev[4], 0));
+  }
+  for (int64_t i = 0; i < chunks && e == cudaSuccess; ++i) {
+    if (i > 0) chk(cudaStreamWaitEvent(s, P->ev[i & 1], 0));
+    if (i + 1 < chunks) {
+      if (i > 0) chk(cudaStreamWaitEvent(side, P->ev[2 + ((i + 1) & 1)], 0));
+      convert(i + 1, side);
+      chk(cudaEventRecord(P->ev[(i + 1) & 1], side));
+    }
+    if (e == cudaSuccess)
+      chk(mlp_place(net, (int)rows_of(i), buf(i), y + 2 * first(i), i + 1 == chunks ? P->y : nullptr,
+                    s));
+    ++P->launches;
+    if (i + 2 < chunks) chk(cudaEventRecord(P->ev[2 + (i & 1)], s));
+  }
+  if (e == cudaSuccess) {
+    P->last_rows = (int)rows_of(chunks - 1);
+    P->pending = true;
+  }
+  return e;
 }
 
 ivhd_status mlp_fail(ivhd_mlp* P, cudaError_t e) {
@@ -753,7 +824,9 @@ ivhd_status ivhd_mlp_set_params(ivhd_mlp* P, const float* params, int32_t on_dev
   if (P->poisoned) return IVHD_ERR_STATE;
   cudaStream_t s = P->stream;
   const size_t bytes = (size_t)P->n_params * sizeof(float);
-  cudaError_t e = cudaMemcpyAsync(P->w, params, bytes,
+  cudaError_t e = hold_activations(P);  // of the last batch, with the weights it used
+  if (e != cudaSuccess) return mlp_fail(P, e);
+  e = cudaMemcpyAsync(P->w, params, bytes,
                                   on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->m, 0, bytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->v, 0, bytes, s);
@@ -795,12 +868,14 @@ ivhd_status ivhd_mlp_train_step(ivhd_mlp* P, const void* x, int32_t x_dtype, flo
   if (!P || !x || !targets || x_dtype < 0 || x_dtype > 2 || !batch_ok(P, B) || !(lr > 0.f))
     return IVHD_ERR_ARG;
   if (P->poisoned) return IVHD_ERR_STATE;
+  P->pending = false;  // this batch replaces the last one
   P->t += 1;
   const float c1 = 1.f - powf(0.9f, (float)P->t), c2 = 1.f - powf(0.999f, (float)P->t);
   cudaError_t e = cudaSuccess;
   if (P->graph_B != B && P->direct_B == B) e = capture_train_step(P, B);
   if (e != cudaSuccess) return mlp_fail(P, e);
   if (P->graph_B == B) {
+    P->last_rows = B;
     e = replay_train_step(P, x, x_dtype, x_scale, targets, B, lr, c1, c2);
   } else {
     // first step at this batch size: run directly (the next one captures it)
@@ -820,6 +895,12 @@ ivhd_status ivhd_mlp_forward(ivhd_mlp* P, const void* x, int32_t x_dtype, float 
   if (P->poisoned) return IVHD_ERR_STATE;
   const size_t esz = x_dtype == 1 ? 1 : (x_dtype == 2 ? 4 : 2);
   cudaError_t e = cudaSuccess;
+  // one kernel per chunk where the hidden width fits tensor memory (it stores
+  // the two outputs of a row at once); otherwise layer by layer
+  if (mlp_place_supported(P->hidden) && (reinterpret_cast<uintptr_t>(y) & 7) == 0) {
+    e = place(P, x, x_dtype, x_scale, n, y);
+    return e != cudaSuccess ? mlp_fail(P, e) : check_err(P);
+  }
   for (int64_t r0 = 0; r0 < n && e == cudaSuccess; r0 += P->max_batch) {
     const int64_t rows = (n - r0 < P->max_batch) ? n - r0 : P->max_batch;
     e = load_x(P, (const char*)x + (size_t)r0 * P->n_in * esz, x_dtype, x_scale, rows);
@@ -837,6 +918,10 @@ int64_t ivhd_mlp_launches(ivhd_mlp* P) { return P ? P->launches : -1; }
 ivhd_status ivhd_mlp_activations(ivhd_mlp* P, int32_t which, void* out, int64_t* rows) {
   if (!P || !out || !rows) return IVHD_ERR_ARG;
   if (P->poisoned) return IVHD_ERR_STATE;
+  if (which == IVHD_MLP_H1 || which == IVHD_MLP_H2) {
+    const cudaError_t e = hold_activations(P);
+    if (e != cudaSuccess) return mlp_fail(P, e);
+  }
   const int64_t B = P->last_rows, H = P->hidden;
   const void* src = nullptr;
   size_t bytes = 0;

@@ -30,8 +30,21 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
                : "r"(addr));
   return v;
 }
+__device__ __forceinline__ void st_shared_u4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c,
+                                             uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
 __device__ __forceinline__ void st_shared_f32(uint32_t addr, float v) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_shared_f2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ float2 ld_shared_f2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ int2 ld_shared_i2(uint32_t addr) {
   int2 v;
@@ -247,6 +260,22 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, 
       "}\n" ::"r"(tmem_d),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
+// `steps` (1 to 4) MMAs of K = 16 on one 64-column slab of A and B; the first
+// overwrites the accumulator when fresh.  One thread issues all MMAs of a
+// pair, so the descriptors are advanced by an addition (a step is 32 bytes, 2 in
+// the descriptor's units) rather than encoded again.
+__device__ __forceinline__ void umma_slab_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                               uint32_t idesc, bool fresh, int steps) {
+  umma_bf16_pair(tmem_d, adesc, bdesc, idesc, fresh ? 0u : 1u);
+  if (steps == 4) {
+    umma_bf16_pair(tmem_d, adesc + 2, bdesc + 2, idesc, 1u);
+    umma_bf16_pair(tmem_d, adesc + 4, bdesc + 4, idesc, 1u);
+    umma_bf16_pair(tmem_d, adesc + 6, bdesc + 6, idesc, 1u);
+    return;
+  }
+  for (int q = 1; q < steps; ++q)
+    umma_bf16_pair(tmem_d, adesc + 2 * q, bdesc + 2 * q, idesc, 1u);
+}
 // Arrives on this barrier in both CTAs once the MMAs issued so far are done.
 __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
   asm volatile(
@@ -258,8 +287,22 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// Bounded wait that also stops when another role of either CTA of a pair has given up.
+__device__ __forceinline__ bool pair_wait(uint64_t* bar, uint32_t parity,
+                                          volatile int* abort_flag) {
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 255u) == 255u && *abort_flag) return false;
+  }
+  for (uint32_t r = 0; r < 2; ++r) st_cluster_u32(pair_addr((const void*)abort_flag, r), 1u);
+  return false;
 }
 
 // Tensor map of a rows x cols BF16 row-major matrix (row stride ld elements):
