@@ -57,11 +57,12 @@ __device__ __forceinline__ float ex2(float x) {
   return r;
 }
 
-// 2^(-a^2 log2(e)/2 + p(a)) = erfc(a / sqrt 2) = 2 Phi(-a) for a = |x|, both values.
-__device__ __forceinline__ float2 erfc_half(F2 x) {
+// 2^(-a^2 log2(e)/2 + p(a)) = erfc(a / sqrt 2) = 2 Phi(-a) for a = |x|, both
+// values; t = min(a, 4 sqrt 2).
+__device__ __forceinline__ float2 erfc_half(F2 x, F2& t) {
   const float2 s = f2_get(x);
   const F2 a = f2(fabsf(s.x), fabsf(s.y));
-  const F2 t = f2(fminf(fabsf(s.x), 5.65685425f), fminf(fabsf(s.y), 5.65685425f));
+  t = f2(fminf(fabsf(s.x), 5.65685425f), fminf(fabsf(s.y), 5.65685425f));
   F2 p = f2_same(4.474227069e-07f);
   p = f2_fma(p, t, f2_same(-8.659556443e-06f));
   p = f2_fma(p, t, f2_same(6.996341108e-05f));
@@ -76,12 +77,13 @@ __device__ __forceinline__ float2 erfc_half(F2 x) {
   return make_float2(ex2(e.x), ex2(e.y));
 }
 
-// GELU of both values.  (The factor a stops at 64, where the exponential has
-// long been zero, so that an infinite x does not meet it as inf * 0.)
+// GELU of both values.  The factor a stops at the end of the polynomial's range
+// too, where the product is below 4e-8 and falling: an infinite x does not meet
+// the exponential's zero as inf * 0.
 __device__ __forceinline__ float2 gelu2(F2 x) {
-  const float2 e = erfc_half(x), s = f2_get(x);
-  const F2 h = f2_mul(f2(fminf(fabsf(s.x), 64.f), fminf(fabsf(s.y), 64.f)), f2_same(-0.5f));
-  return f2_get(f2_fma(h, f2(e.x, e.y), f2(fmaxf(s.x, 0.f), fmaxf(s.y, 0.f))));
+  F2 t;
+  const float2 e = erfc_half(x, t), s = f2_get(x);
+  return f2_get(f2_fma(f2_mul(t, f2_same(-0.5f)), f2(e.x, e.y), f2(fmaxf(s.x, 0.f), fmaxf(s.y, 0.f))));
 }
 
 }  // namespace ivhd

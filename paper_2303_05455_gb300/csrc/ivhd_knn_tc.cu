@@ -31,21 +31,21 @@
 //
 // A pair of CTAs (a cluster of two, cta_group::2) owns 256 query rows, 128
 // tensor-memory lanes each, and sweeps all candidates in tiles of 256 columns:
-//   warp 0, one lane   TMA producer: this CTA's 128 x 64 query slice and its
-//                      half (128 x 64) of the candidate slice into a 6-stage
+//   warps 0, 10        TMA producers: this CTA's 128 x 64 query slice, and its
+//                      half (128 x 64) of the candidate slice, into a 6-stage
 //                      ring (128-byte swizzle); 32 KB from L2 per 512 clocks of
-//                      MMAs instead of 48 KB with a tile per CTA
-//   warp 1, one lane   (rank 0) MMA issuer: tcgen05.mma M=256 N=256 K=16 into one
+//                      MMAs instead of 48 KB with a tile per CTA (one warp's
+//                      copies reach about 50 bytes per clock, two warps' 93)
+//   warp 1             (rank 0) MMA issuer: tcgen05.mma M=256 N=256 K=16 into one
 //                      of two 256-column accumulators in tensor memory, so the
 //                      epilogue of tile t overlaps the MMAs of tile t+1
 //   warps 2-9          epilogue: thread = query row; tcgen05.ld of 16 columns at
 //                      a time, distance, test against the row's threshold, a
 //                      queue in shared memory and a list in registers
 // Every wait is bounded; a timeout sets an error flag and all roles stop.
-// What bounds it (kernel alone, M = 100,000 floats x 100, K = 320): 3.6 ms with
-// the epilogue doing nothing (1.77 PFLOP/s, the tensor cores at their power
-// limit), 3.7 ms with its tests but no candidate passing; handling the
-// candidates takes the rest.
+// What bounds it: float, handling the candidates that pass (with one producer,
+// M = 100,000 x 100, K = 320: 3.6 ms with the epilogue doing nothing, 3.7 ms
+// with its tests but no candidate passing, 5 ms in all); uint8, the MMAs.
 #include <climits>
 #include <cstdint>
 #include <cstring>
@@ -64,7 +64,7 @@ constexpr int kTM = 128;  // query rows per CTA (two CTAs share a 256-row tile)
 constexpr int kTN = 256;  // candidate columns per accumulator tile, half of them loaded by each CTA
 constexpr int kTStages = 6;
 constexpr int kEpiWarps = 8;  // two warpgroups: each reads one 128-column half of a tile
-constexpr int kTcThreads = 32 * (2 + kEpiWarps);
+constexpr int kTcThreads = 32 * (3 + kEpiWarps);
 constexpr int kMaxKnnSegments = 32;  // column segments of one kNN launch (short query sets)
 constexpr int kGroup = 8;            // columns tested and queued together in the epilogue
 constexpr int kChunk = 16;           // columns read from tensor memory at once
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   constexpr uint32_t kCols = 2 * kTN;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cta_rank();  // 0: the CTA that issues the MMAs of the pair
   const int m0 = blockIdx.x * kTM;
   const int nk = Kp / kBK;
@@ -174,69 +174,73 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
-    if (lane == 0) {
-      // producer: this CTA's query slice (re-read from L2 for every tile) and
-      // its half of the candidate slice; the bytes of both CTAs are counted by
-      // the barrier of rank 0
-      uint32_t g = 0;
-      bool ok = true;
-      for (int t = 0; t < n_tiles && ok; ++t) {
-        for (int kt = 0; kt < nk; ++kt, ++g) {
-          const int s = (int)(g % kTStages);
-          if (g >= kTStages && !pair_wait(&empty[s], ((g / kTStages) - 1) & 1, abort_flag)) {
-            atomicOr(err, 1);
-            ok = false;
-            break;
-          }
-          unsigned char* sa = smem + s * KnnSmem::stage_bytes;
-          unsigned char* sb = sa + KnnSmem::a_bytes;
-          if (rank == 0) mbar_expect_tx(&full[s], 2 * KnnSmem::stage_bytes);
-          const uint32_t bar = pair_addr(&full[s], 0);
-          tma_load_2d_pair(sa, &map_a, kt * kBK, m0, bar);
-          tma_load_2d_pair(sb, &map_b, kt * kBK, (t0 + t) * kTN + (int)rank * (kTN / 2), bar);
+  if (warp == 0 || warp == 2 + kEpiWarps) {
+    // producers: this CTA's query slice (re-read from L2 for every tile), and its
+    // half of the candidate slice; the bytes of both CTAs are counted by the
+    // barrier of rank 0
+    const bool second = warp != 0;
+    const uint32_t full0 = pair_addr(full, 0);
+    int s = 0;
+    uint32_t lap = 0;
+    bool ok = true;
+    for (int t = 0; t < n_tiles && ok; ++t) {
+      const int y = second ? (t0 + t) * kTN + (int)rank * (kTN / 2) : m0;
+      for (int kt = 0; kt < nk; ++kt) {
+        if (lap > 0) ok = __all_sync(0xffffffffu, pair_wait(&empty[s], (lap - 1) & 1, abort_flag));
+        if (!ok) break;
+        if (elect_one()) {
+          if (rank == 0 && !second) mbar_expect_tx(&full[s], 2 * KnnSmem::stage_bytes);
+          tma_load_2d_pair(smem + s * KnnSmem::stage_bytes + (second ? KnnSmem::a_bytes : 0),
+                           second ? &map_b : &map_a, kt * kBK, y, full0 + (uint32_t)s * 8u);
+        }
+        if (++s == kTStages) {
+          s = 0;
+          ++lap;
         }
       }
+    }
+    if (!ok) {
+      if (lane == 0) atomicOr(err, 1);
       // a copy in flight lands within microseconds: after an abort, time for
       // it before the shared memory goes away
-      if (!ok)
-        for (int it = 0; it < 2000; ++it) __nanosleep(1000);
+      for (int it = 0; it < 2000; ++it) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = instr_desc_bf16(2 * kTM, kTN);
-      uint32_t g = 0;
+      const uint64_t desc = smem_desc_sw128(smem_u32(smem));
+      int s = 0;
+      uint32_t lap = 0;
       bool ok = true;
+      auto wait = [&](uint64_t* bar, uint32_t parity, int code) {
+        ok = __all_sync(0xffffffffu, pair_wait(bar, parity, abort_flag));
+        if (!ok && lane == 0) atomicOr(err, code);
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        return ok;
+      };
       for (int t = 0; t < n_tiles && ok; ++t) {
         const int b = t & 1;
-        if (t >= 2 && !pair_wait(&acc_empty[b], ((t >> 1) - 1) & 1, abort_flag)) {
-          atomicOr(err, 2);
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (t >= 2 && !wait(&acc_empty[b], ((t >> 1) - 1) & 1, 2)) break;
         const uint32_t dst = tmem + (uint32_t)(b * kTN);
-        for (int kt = 0; kt < nk; ++kt, ++g) {
-          const int s = (int)(g % kTStages);
-          if (!pair_wait(&full[s], (g / kTStages) & 1, abort_flag)) {
-            atomicOr(err, 4);
-            ok = false;
-            break;
+        for (int kt = 0; kt < nk; ++kt) {
+          if (!wait(&full[s], lap & 1, 4)) break;
+          if (elect_one()) {
+            const uint64_t a = desc + (uint64_t)(s * (KnnSmem::stage_bytes >> 4));
+            umma_slab_pair(dst, a, a + (KnnSmem::a_bytes >> 4), idesc, kt == 0, kBK / 16);
+            umma_commit_pair(&empty[s]);
+            if (kt + 1 == nk) umma_commit_pair(&acc_full[b]);
           }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const uint32_t sa = smem_u32(smem + s * KnnSmem::stage_bytes);
-          const uint32_t sb = sa + KnnSmem::a_bytes;
-#pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk)
-            umma_bf16_pair(dst, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32),
-                           idesc, (kt > 0 || kk > 0) ? 1u : 0u);
-          umma_commit_pair(&empty[s]);
+          __syncwarp();
+          if (++s == kTStages) {
+            s = 0;
+            ++lap;
+          }
         }
-        if (ok) umma_commit_pair(&acc_full[b]);
       }
       // every MMA issued above has finished before tensor memory is released
       // and either CTA's shared memory goes away
-      umma_commit_pair(done);
-      if (!mbar_wait(done, 0)) atomicOr(err, 8);
+      if (elect_one()) umma_commit_pair(done);
+      if (!mbar_wait(done, 0) && lane == 0) atomicOr(err, 8);
     }
   } else {
     // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. 32 (w % 4) + 31
@@ -253,7 +257,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // at once made the whole warp walk one row's list, and that, not the tensor
     // cores, set the time (whole build, 300,000 x 100 floats, k = 5: 70.4 -> 44.2 ms
     // with queues, 42.7 with appends that do not branch, loads that run ahead and
-    // shared bounds; 70,000 x 784 bytes 6.00 -> 5.59 -> 5.01 ms).
+    // shared bounds, 38.8 with the second producer; 70,000 x 784 bytes 6.00 ->
+    // 5.59 -> 5.01 -> 4.44 ms).
     // uint8: the float key and the float threshold are within 2 of the exact
     // integers (magnitudes below 2^26), so the test allows 16 and the queue takes
     // the exact keys.

@@ -7,7 +7,7 @@
 // output layer's sum runs in another fixed order).  The activations never
 // leave the SM: a layer at a time wrote and re-read 2 KB per row, and its GEMMs
 // were bound by that epilogue.  1.4e6 rows of 784 bytes, hidden 512: 5.63 ms
-// layer by layer, 2.56 ms here (the MMAs need 1.0 ms at the tensor cores' rate).
+// layer by layer, 2.36 ms here (the MMAs need 1.0 ms at the tensor cores' rate).
 //
 // A pair of CTAs (cta_group::2) takes 256 rows at a time, 128 each, and loops
 // over such tiles (persistent).  The hidden layers are computed in chunks of
@@ -25,6 +25,8 @@
 //   warp 1      MMA issuer (rank 0)
 //   warps 2-17  epilogue: four warps per tensor-memory lane quadrant, a quarter
 //               of the chunk's columns each
+//   warp 18     TMA: the second slab of every stage (copies issued by one warp
+//               reach about 50 bytes per clock, by two about 93)
 // Waits are bounded; on timeout an error flag is raised and all roles stop.
 #include "ivhd_gelu.cuh"
 #include "ivhd_gemm.cuh"
@@ -45,7 +47,7 @@ constexpr int kStage = 2 * kSlab;      // layer 1: x and W1; layer 2: two slabs 
 constexpr int kStages = 3;
 constexpr int kParts = 4;              // column quarters of a chunk
 constexpr int kEpi = 4 * kParts;       // epilogue warps
-constexpr int kThreads = 32 * (2 + kEpi);
+constexpr int kThreads = 32 * (3 + kEpi);
 
 // Shared memory: the layer-1 activations (up to 128 KB), the ring, the barriers.
 __host__ __device__ constexpr int h1_slabs(int H) { return (H + kBK - 1) / kBK; }
@@ -88,7 +90,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cta_rank();
   const int pair = (int)blockIdx.x >> 1, n_pairs = (int)gridDim.x >> 1;
   const int n_tiles = (rows + 2 * kRows - 1) / (2 * kRows);
@@ -134,50 +136,47 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   };
 
-  if (warp == 0) {
-    if (lane == 0) {
-      Cursor c;
-      bool ok = true;
-      const uint32_t full0 = pair_addr(full, 0);
-      // a stage of one or two slabs
-      auto load = [&](const CUtensorMap* ma, int xa, int ya, const CUtensorMap* mb, int xb, int yb) {
-        if (c.lap > 0 && !pair_wait(&empty[c.s], (c.lap - 1) & 1, abort_flag)) {
-          atomicOr(err, 1);
-          ok = false;
-          return;
-        }
-        if (rank == 0) mbar_expect_tx(&full[c.s], 2 * (mb ? kStage : kSlab));
-        const uint32_t bar = full0 + (uint32_t)c.s * 8u;
-        tma_load_2d_pair(ring + c.s * kStage, ma, xa, ya, bar);
-        if (mb) tma_load_2d_pair(ring + c.s * kStage + kSlab, mb, xb, yb, bar);
-        c.next();
-      };
-      for (int t = pair; t < n_tiles && ok; t += n_pairs) {
-        const int row = (2 * t + (int)rank) * kRows;
-        for (int n = 0; n < nc && ok; ++n) {
-          const int w = n * kChunkN + (int)rank * (width(n) / 2);
-          for (int k = 0; k < nk1 && ok; ++k) load(&map_x, k * kBK, row, &map_w1, k * kBK, w);
-        }
-        for (int n = 0; n < nc && ok; ++n) {
-          const int w = n * kChunkN + (int)rank * (width(n) / 2);
-          for (int k = 0; k < nk2 && ok; k += 2)
-            load(&map_w2, k * kBK, w, k + 1 < nk2 ? &map_w2 : nullptr, (k + 1) * kBK, w);
-        }
+  if (warp == 0 || warp == 2 + kEpi) {
+    // the first and the second slab of every stage; the first producer of rank 0
+    // announces the bytes of all
+    const int second = warp != 0;
+    Cursor c;
+    bool ok = true;
+    const uint32_t full0 = pair_addr(full, 0);
+    auto load = [&](const CUtensorMap* map, int x, int y, int slabs) {
+      if (c.lap > 0) ok = __all_sync(0xffffffffu, pair_wait(&empty[c.s], (c.lap - 1) & 1, abort_flag));
+      if (!ok) return;
+      if (elect_one()) {
+        if (rank == 0 && !second) mbar_expect_tx(&full[c.s], 2 * slabs * kSlab);
+        if (second < slabs)
+          tma_load_2d_pair(ring + c.s * kStage + second * kSlab, map, x, y, full0 + (uint32_t)c.s * 8u);
       }
+      c.next();
+    };
+    for (int t = pair; t < n_tiles && ok; t += n_pairs) {
+      for (int n = 0; n < nc && ok; ++n) {
+        const int y = second ? n * kChunkN + (int)rank * (width(n) / 2) : (2 * t + (int)rank) * kRows;
+        for (int k = 0; k < nk1 && ok; ++k) load(second ? &map_w1 : &map_x, k * kBK, y, 2);
+      }
+      for (int n = 0; n < nc && ok; ++n) {
+        const int y = n * kChunkN + (int)rank * (width(n) / 2);
+        for (int k = 0; k < nk2 && ok; k += 2)
+          load(&map_w2, (k + second) * kBK, y, min(2, nk2 - k));
+      }
+    }
+    if (!ok) {
+      if (lane == 0) atomicOr(err, 1);
       // a copy in flight lands within microseconds: after an abort, time for
       // it before the shared memory goes away
-      if (!ok)
-        for (int it = 0; it < 2000; ++it) __nanosleep(1000);
+      for (int it = 0; it < 2000; ++it) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       Cursor c;
       bool ok = true;
       auto wait = [&](uint64_t* bar, uint32_t parity, int code) {
-        if (ok && !pair_wait(bar, parity, abort_flag)) {
-          atomicOr(err, code);
-          ok = false;
-        }
+        ok = __all_sync(0xffffffffu, pair_wait(bar, parity, abort_flag));
+        if (!ok && lane == 0) atomicOr(err, code);
         asm volatile("tcgen05.fence::after_thread_sync;");
         return ok;
       };
@@ -189,12 +188,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t dst = tmem + (uint32_t)(n * kChunkN), idesc = instr_desc_bf16(2 * kRows, width(n));
           for (int k = 0; k < nk1; ++k) {
             if (!wait(&full[c.s], c.lap & 1, 2)) break;
-            const uint64_t a = ring_desc + (uint64_t)(c.s * (kStage >> 4));
-            umma_slab_pair(dst, a, a + (kSlab >> 4), idesc, k == 0, min(kBK / 16, (n_in - k * kBK + 15) / 16));
-            umma_commit_pair(&empty[c.s]);
+            if (elect_one()) {
+              const uint64_t a = ring_desc + (uint64_t)(c.s * (kStage >> 4));
+              umma_slab_pair(dst, a, a + (kSlab >> 4), idesc, k == 0, min(kBK / 16, (n_in - k * kBK + 15) / 16));
+              umma_commit_pair(&empty[c.s]);
+              if (k + 1 == nk1) umma_commit_pair(&acc_full[n]);
+            }
+            __syncwarp();
             c.next();
           }
-          if (ok) umma_commit_pair(&acc_full[n]);
         }
         for (int n = 0; n < nc && ok; ++n) {
           const uint32_t dst = tmem + (uint32_t)(n * kChunkN), idesc = instr_desc_bf16(2 * kRows, width(n));
@@ -203,20 +205,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             // chunk also frees its accumulator)
             if (n == 0 && k % (kChunkN / kBK) == 0 && !wait(&acc_done[k / (kChunkN / kBK)], 0, 8)) break;
             if (!wait(&full[c.s], c.lap & 1, 2)) break;
-            const uint64_t b = ring_desc + (uint64_t)(c.s * (kStage >> 4));
-            const uint64_t a = h1_desc + (uint64_t)(k * (kSlab >> 4));
-            umma_slab_pair(dst, a, b, idesc, k == 0, min(kBK / 16, (H - k * kBK) / 16));
-            if (k + 1 < nk2)
-              umma_slab_pair(dst, a + (kSlab >> 4), b + (kSlab >> 4), idesc, false,
-                             min(kBK / 16, (H - (k + 1) * kBK) / 16));
-            umma_commit_pair(&empty[c.s]);
+            if (elect_one()) {
+              const uint64_t b = ring_desc + (uint64_t)(c.s * (kStage >> 4));
+              const uint64_t a = h1_desc + (uint64_t)(k * (kSlab >> 4));
+              umma_slab_pair(dst, a, b, idesc, k == 0, min(kBK / 16, (H - k * kBK) / 16));
+              if (k + 1 < nk2)
+                umma_slab_pair(dst, a + (kSlab >> 4), b + (kSlab >> 4), idesc, false,
+                               min(kBK / 16, (H - (k + 1) * kBK) / 16));
+              umma_commit_pair(&empty[c.s]);
+              if (k + 2 >= nk2) umma_commit_pair(&acc_full[n]);
+            }
+            __syncwarp();
             c.next();
           }
-          if (ok) umma_commit_pair(&acc_full[n]);
         }
       }
-      umma_commit_pair(done);
-      if (!mbar_wait(done, 0)) atomicOr(err, 16);
+      if (elect_one()) umma_commit_pair(done);
+      if (!mbar_wait(done, 0) && lane == 0) atomicOr(err, 16);
     }
   } else {
     const int quarter = warp & 3, part = (warp - 2) >> 2;

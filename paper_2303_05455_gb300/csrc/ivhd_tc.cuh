@@ -224,6 +224,26 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
 // accumulator in its tensor memory; one thread of the CTA of rank 0 issues
 // the MMAs for both.
 
+// One lane of a converged warp.  The issuing warps run their loops with all
+// lanes and elect one per instruction: positions and descriptors then stay in
+// uniform registers, which the MMA and TMA instructions read; from a branch on
+// the lane index every operand was moved there again for every instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.b32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(p));
+  return p != 0;
+}
+// The warp's index, the same register for all its lanes.
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+}
+
 __device__ __forceinline__ uint32_t cta_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
