@@ -86,4 +86,16 @@ __device__ __forceinline__ float2 gelu2(F2 x) {
   return f2_get(f2_fma(f2_mul(t, f2_same(-0.5f)), f2(e.x, e.y), f2(fmaxf(s.x, 0.f), fmaxf(s.y, 0.f))));
 }
 
+// GELU'(x) = Phi(x) + x phi(x) of both values.
+__device__ __forceinline__ float2 gelu_grad2(F2 x) {
+  F2 t;
+  const float2 e = erfc_half(x, t), s = f2_get(x);
+  // Phi = 1/2 + copysign(1/2 - Phi(-a), x)
+  const float2 c = f2_get(f2_fma(f2(e.x, e.y), f2_same(-0.5f), f2_same(0.5f)));
+  const F2 cdf = f2_add(f2(copysignf(c.x, s.x), copysignf(c.y, s.y)), f2_same(0.5f));
+  const float2 g = f2_get(f2_mul(f2_mul(x, f2_same(-0.72134752044448170f)), x));
+  const F2 pdf = f2_mul(f2(ex2(g.x), ex2(g.y)), f2_same(0.39894228040143268f));
+  return f2_get(f2_fma(x, pdf, cdf));
+}
+
 }  // namespace ivhd

@@ -6,12 +6,15 @@
 // carries the dense layers of the learned warm start (an MLP that maps features
 // to 2-D positions, trained on IVHD embeddings).
 //
-// Persistent kernel, one CTA per SM, looping over 128 x BN output tiles
-// (BN = 256, or 128 when that keeps more SMs busy or pads N less):
-//   warp 0, one lane   TMA producer: 128 x 64 A and BN x 64 B tiles into a
+// Persistent kernel, looping over 128 x BN output tiles, one CTA per SM (BN = 256,
+// or 128 when that keeps more SMs busy or pads N less) or two (BN = 64, for
+// products of few tiles: their time is the epilogue's, and twice the warps work
+// on it; batch 4,096, hidden 512, under ncu: W1 forward 20.5 -> 17.0 us, W2
+// forward 17.0 -> 14.0, dH 18.2 -> 15.5, dW1 16.3 -> 12.9):
+//   warps 0, 10        TMA producers: 128 x 64 A and BN x 64 B tiles into a
 //                      4- or 6-stage shared-memory ring (128-byte swizzle), one
 //                      mbarrier with a transaction count per stage
-//   warp 1, one lane   MMA issuer: four tcgen05.mma (K = 16 each) per stage into
+//   warp 1             MMA issuer: four tcgen05.mma (K = 16 each) per stage into
 //                      one of two tensor-memory accumulators; tcgen05.commit
 //                      frees the stage, a commit per tile hands the
 //                      accumulator to the epilogue
@@ -30,6 +33,7 @@
 #include <mutex>
 #include <unordered_map>
 
+#include "ivhd_gelu.cuh"
 #include "ivhd_gemm.cuh"
 #include "ivhd_internal.cuh"
 #include "ivhd_tc.cuh"
@@ -119,60 +123,53 @@ using namespace tc;
 
 constexpr int kBM = 128;
 constexpr int kEpiWarps = 8;       // two per tensor-memory lane quadrant, each half the columns
-constexpr int kGemmThreads = 32 * (2 + kEpiWarps);  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
-
-__device__ __forceinline__ float gelu(float x) {
-  return 0.5f * x * (1.f + erff(x * 0.70710678118654752f));
-}
-__device__ __forceinline__ float gelu_grad(float x) {
-  const float cdf = 0.5f * (1.f + erff(x * 0.70710678118654752f));
-  const float pdf = 0.39894228040143268f * expf(-0.5f * x * x);
-  return cdf + x * pdf;
-}
+constexpr int kGemmThreads = 32 * (3 + kEpiWarps);  // warps 0, 10 TMA, warp 1 MMA, warps 2-9 epilogue
 
 __device__ __forceinline__ bool aligned16(const void* p) {
   return (reinterpret_cast<uintptr_t>(p) & 15) == 0;
 }
 
-// 32 BF16 values (round to nearest even) stored as four 16-byte words.
-__device__ __forceinline__ void store_bf16x32(__nv_bfloat16* o, const float* t) {
-  uint32_t w[16];
+constexpr int kCols = 16;  // accumulator columns handled at once: 8 pairs for the packed FP32 pipe
+
+// kCols BF16 values (round to nearest even) stored as 16-byte words.
+__device__ __forceinline__ void store_bf16(__nv_bfloat16* o, const float* t) {
+  uint32_t w[kCols / 2];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < kCols / 2; ++q) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(t[2 * q], t[2 * q + 1]);
     memcpy(&w[q], &h, 4);
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < kCols / 8; ++q)
     reinterpret_cast<uint4*>(o)[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
 }
 
-// The transposed copy of 32 BF16 values of one row: column col0 + q of this
+// The transposed copy of kCols BF16 values of one row: column col0 + q of this
 // row goes to out_t[(col0 + q) * ld_t + row].  The lanes of a warp hold
-// consecutive rows, so each of the 32 stores is one contiguous 64-byte run.
+// consecutive rows, so each store is one contiguous 64-byte run.
 __device__ __forceinline__ void store_bf16_t(__nv_bfloat16* out_t, int64_t ld_t, int row,
                                              int col0, int N, const float* t) {
 #pragma unroll
-  for (int q = 0; q < 32; ++q)
+  for (int q = 0; q < kCols; ++q)
     if (col0 + q < N) out_t[(int64_t)(col0 + q) * ld_t + row] = __float2bfloat16_rn(t[q]);
 }
 
-// Epilogue of 32 consecutive accumulator columns of one row: v[q] = C[row, col0 + q].
-// Vector stores where the 32 columns are in range and 16-byte aligned, else
+// Epilogue of kCols consecutive accumulator columns of one row: v[q] = C[row, col0 + q].
+// Vector accesses where the columns are in range and 16-byte aligned, else
 // element by element; the value written per element is the same either way.
-__device__ __forceinline__ void ep_apply32(const GemmEpilogue& ep, int row, int col0, int N,
-                                           const float* v) {
+__device__ __forceinline__ void ep_apply(const GemmEpilogue& ep, int row, int col0, int N,
+                                         const float* v) {
   const int64_t off = (int64_t)row * ep.ld_out + col0;
-  const bool full = col0 + 32 <= N;
+  const bool full = col0 + kCols <= N;
   if (ep.kind == kEpStoreF32) {
     float* o = ep.out_f32 + off;
     if (full && aligned16(o)) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
+      for (int q = 0; q < kCols / 4; ++q)
         reinterpret_cast<float4*>(o)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     } else {
 #pragma unroll
-      for (int q = 0; q < 32; ++q)
+      for (int q = 0; q < kCols; ++q)
         if (col0 + q < N) o[q] = v[q];
     }
   } else if (ep.kind == kEpBiasGelu) {
@@ -180,23 +177,35 @@ __device__ __forceinline__ void ep_apply32(const GemmEpilogue& ep, int row, int 
     // given: training); h = GELU(z) in BF16
     float* z = ep.out_f32 ? ep.out_f32 + off : nullptr;
     __nv_bfloat16* h = ep.out_bf16 + off;
-    float t[32], g[32];
+    float t[kCols], g[kCols];
+    const bool vec_bias = full && aligned16(ep.bias + col0);
 #pragma unroll
-    for (int q = 0; q < 32; ++q) {
-      t[q] = (col0 + q < N) ? v[q] + ep.bias[col0 + q] : 0.f;
-      g[q] = gelu(t[q]);
+    for (int q = 0; q < kCols; q += 4) {
+      float4 b;
+      if (vec_bias) {
+        b = __ldg(reinterpret_cast<const float4*>(ep.bias + col0 + q));
+      } else {
+        b.x = col0 + q < N ? ep.bias[col0 + q] : 0.f;
+        b.y = col0 + q + 1 < N ? ep.bias[col0 + q + 1] : 0.f;
+        b.z = col0 + q + 2 < N ? ep.bias[col0 + q + 2] : 0.f;
+        b.w = col0 + q + 3 < N ? ep.bias[col0 + q + 3] : 0.f;
+      }
+      const F2 z0 = f2_add(f2(v[q], v[q + 1]), f2(b.x, b.y)), z1 = f2_add(f2(v[q + 2], v[q + 3]), f2(b.z, b.w));
+      const float2 t0 = f2_get(z0), t1 = f2_get(z1), g0 = gelu2(z0), g1 = gelu2(z1);
+      t[q] = t0.x, t[q + 1] = t0.y, t[q + 2] = t1.x, t[q + 3] = t1.y;
+      g[q] = g0.x, g[q + 1] = g0.y, g[q + 2] = g1.x, g[q + 3] = g1.y;
     }
     if (full && (!z || aligned16(z)) && aligned16(h)) {
       if (z) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
+        for (int q = 0; q < kCols / 4; ++q)
           reinterpret_cast<float4*>(z)[q] =
               make_float4(t[4 * q], t[4 * q + 1], t[4 * q + 2], t[4 * q + 3]);
       }
-      store_bf16x32(h, g);
+      store_bf16(h, g);
     } else {
 #pragma unroll
-      for (int q = 0; q < 32; ++q)
+      for (int q = 0; q < kCols; ++q)
         if (col0 + q < N) {
           if (z) z[q] = t[q];
           h[q] = __float2bfloat16_rn(g[q]);
@@ -207,10 +216,10 @@ __device__ __forceinline__ void ep_apply32(const GemmEpilogue& ep, int row, int 
     // dZ = acc * GELU'(z) in BF16 (acc is dH)
     const float* z = ep.aux_f32 + off;
     __nv_bfloat16* o = ep.out_bf16 + off;
-    float zz[32], t[32];
+    float zz[kCols], t[kCols];
     if (full && aligned16(z)) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < kCols / 4; ++q) {
         const float4 f = reinterpret_cast<const float4*>(z)[q];
         zz[4 * q] = f.x;
         zz[4 * q + 1] = f.y;
@@ -219,19 +228,33 @@ __device__ __forceinline__ void ep_apply32(const GemmEpilogue& ep, int row, int 
       }
     } else {
 #pragma unroll
-      for (int q = 0; q < 32; ++q) zz[q] = (col0 + q < N) ? z[q] : 0.f;
+      for (int q = 0; q < kCols; ++q) zz[q] = (col0 + q < N) ? z[q] : 0.f;
     }
 #pragma unroll
-    for (int q = 0; q < 32; ++q) t[q] = v[q] * gelu_grad(zz[q]);
+    for (int q = 0; q < kCols; q += 2) {
+      const float2 g = gelu_grad2(f2(zz[q], zz[q + 1]));
+      t[q] = v[q] * g.x;
+      t[q + 1] = v[q + 1] * g.y;
+    }
     if (full && aligned16(o)) {
-      store_bf16x32(o, t);
+      store_bf16(o, t);
     } else {
 #pragma unroll
-      for (int q = 0; q < 32; ++q)
+      for (int q = 0; q < kCols; ++q)
         if (col0 + q < N) o[q] = __float2bfloat16_rn(t[q]);
     }
     if (ep.out_bf16_t) store_bf16_t(ep.out_bf16_t, ep.ld_t, row, col0, N, t);
   }
+}
+
+// Bounded wait that also stops when another role has given up.
+__device__ __forceinline__ bool wait_or_stop(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 255u) == 255u && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
 }
 
 template <int BN, int STAGES>
@@ -241,6 +264,8 @@ struct GemmSmem {
   static constexpr int stage_bytes = a_bytes + b_bytes;
   static constexpr int bar_offset = STAGES * stage_bytes;
   static constexpr int total = bar_offset + 256 + 1024;  // + alignment slack
+  // CTAs per SM: two where shared memory and tensor memory hold both
+  static constexpr int per_sm = 2 * total <= 227 * 1024 && 4 * BN <= 512 ? 2 : 1;
 };
 
 // A work unit: output tile (tm, tn) and split-K slice z with its k-tiles
@@ -275,7 +300,7 @@ __device__ __forceinline__ Unit unit_of(int u, int tiles_m, int tiles_n, int spl
 //   acc_full[b]             accumulator b complete (MMA commit)
 //   acc_empty[b]            accumulator b read out (one arrival per epilogue warp)
 template <int BN, int STAGES>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kGemmThreads, GemmSmem<BN, STAGES>::per_sm)
     k_gemm_bf16_tn(const __grid_constant__ CUtensorMap map_a,
                    const __grid_constant__ CUtensorMap map_b, GemmEpilogue ep, int M, int N,
                    int K, int splits, int32_t* __restrict__ err) {
@@ -286,12 +311,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint64_t* empty = full + STAGES;
   uint64_t* acc_full = empty + STAGES;
   uint64_t* acc_empty = acc_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* done = acc_empty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* issued = abort_flag + 1;  // k-tile loads issued (for the drain after an abort)
   constexpr uint32_t kTmemCols = 2 * BN;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int tiles_m = (M + kBM - 1) / kBM, tiles_n = (N + BN - 1) / BN;
   const int nk_all = (K + kBK - 1) / kBK;
   const int units = tiles_m * tiles_n * splits;
@@ -305,8 +330,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       mbar_init(&acc_full[b], 1);
       mbar_init(&acc_empty[b], kEpiWarps);
     }
+    mbar_init(done, 1);
     *abort_flag = 0;
-    *issued = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -320,66 +345,76 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
-    if (lane == 0) {
-      // TMA producer
-      int it = 0;
-      for (int u = blockIdx.x; u < units && !*abort_flag; u += gridDim.x) {
-        const Unit w = unit_of(u, tiles_m, tiles_n, splits, nk_all);
-        for (int kt = 0; kt < w.nk; ++kt, ++it) {
-          const int s = it % STAGES;
-          if (it >= STAGES && !mbar_wait(&empty[s], ((it / STAGES) - 1) & 1)) {
-            atomicOr(err, 1);
-            *abort_flag = 1;
-            break;
-          }
-          if (*abort_flag) break;
-          unsigned char* sa = smem + s * S::stage_bytes;
-          unsigned char* sb = sa + S::a_bytes;
-          mbar_expect_tx(&full[s], S::stage_bytes);
-          tma_load_2d(sa, &map_a, (w.kt0 + kt) * kBK, w.tm * kBM, &full[s]);
-          tma_load_2d(sb, &map_b, (w.kt0 + kt) * kBK, w.tn * BN, &full[s]);
-          *issued = it + 1;
+  if (warp == 0 || warp == 2 + kEpiWarps) {
+    // TMA producers, one for each operand (one warp's copies reach about 50
+    // bytes per clock, two warps' 93); the first announces the bytes of both
+    const bool second = warp != 0;
+    int s = 0;
+    uint32_t lap = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      const Unit w = unit_of(u, tiles_m, tiles_n, splits, nk_all);
+      const int y = second ? w.tn * BN : w.tm * kBM;
+      for (int kt = 0; kt < w.nk; ++kt) {
+        if (lap > 0) ok = __all_sync(0xffffffffu, wait_or_stop(&empty[s], (lap - 1) & 1, abort_flag));
+        if (!ok) break;
+        if (elect_one()) {
+          if (!second) mbar_expect_tx(&full[s], S::stage_bytes);
+          tma_load_2d(smem + s * S::stage_bytes + (second ? S::a_bytes : 0), second ? &map_b : &map_a,
+                      (w.kt0 + kt) * kBK, y, &full[s]);
+        }
+        if (++s == STAGES) {
+          s = 0;
+          ++lap;
         }
       }
+    }
+    if (!ok) {
+      if (lane == 0) atomicOr(err, 1);
+      // a copy in flight lands within microseconds: after an abort, time for
+      // it before the shared memory goes away
+      for (int it = 0; it < 2000; ++it) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      constexpr uint32_t idesc = instr_desc_bf16(kBM, BN);
-      int it = 0, j = 0;
-      for (int u = blockIdx.x; u < units && !*abort_flag; u += gridDim.x, ++j) {
-        const Unit w = unit_of(u, tiles_m, tiles_n, splits, nk_all);
-        const int b = j & 1;
-        if (j >= 2 && !mbar_wait(&acc_empty[b], ((j >> 1) - 1) & 1)) {
-          atomicOr(err, 8);
-          *abort_flag = 1;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t d = tmem + (uint32_t)(b * BN);
-        bool ok = true;
-        for (int kt = 0; kt < w.nk; ++kt, ++it) {
-          const int s = it % STAGES;
-          if (!mbar_wait(&full[s], (it / STAGES) & 1)) {
-            atomicOr(err, 2);
-            *abort_flag = 1;
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const uint32_t sa = smem_u32(smem + s * S::stage_bytes);
-          const uint32_t sb = sa + S::a_bytes;
+    // MMA issuer
+    constexpr uint32_t idesc = instr_desc_bf16(kBM, BN);
+    const uint64_t desc = smem_desc_sw128(smem_u32(smem));
+    int s = 0, j = 0;
+    uint32_t lap = 0;
+    bool ok = true;
+    auto wait = [&](uint64_t* bar, uint32_t parity, int code) {
+      ok = __all_sync(0xffffffffu, wait_or_stop(bar, parity, abort_flag));
+      if (!ok && lane == 0) atomicOr(err, code);
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      return ok;
+    };
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++j) {
+      const Unit w = unit_of(u, tiles_m, tiles_n, splits, nk_all);
+      const int b = j & 1;
+      if (j >= 2 && !wait(&acc_empty[b], ((j >> 1) - 1) & 1, 8)) break;
+      const uint32_t d = tmem + (uint32_t)(b * BN);
+      for (int kt = 0; kt < w.nk; ++kt) {
+        if (!wait(&full[s], lap & 1, 2)) break;
+        if (elect_one()) {
+          const uint64_t da = desc + (uint64_t)(s * (S::stage_bytes >> 4)), db = da + (S::a_bytes >> 4);
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk)
-            umma_bf16(d, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32), idesc,
-                      (kt > 0 || kk > 0) ? 1u : 0u);
+            umma_bf16(d, da + 2 * kk, db + 2 * kk, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
           umma_commit(&empty[s]);
         }
-        if (!ok) break;
-        umma_commit(&acc_full[b]);  // this unit's MMAs (an empty slice arrives at once)
+        __syncwarp();
+        if (++s == STAGES) {
+          s = 0;
+          ++lap;
+        }
       }
+      // this unit's MMAs (an empty slice arrives at once)
+      if (ok && elect_one()) umma_commit(&acc_full[b]);
+      __syncwarp();
     }
+    // every MMA issued above has finished before tensor memory is released
+    if (elect_one()) umma_commit(done);
+    if (!mbar_wait(done, 0) && lane == 0) atomicOr(err, 16);
   } else {
     // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31
     const int q = warp & 3;
@@ -389,31 +424,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const Unit w = unit_of(u, tiles_m, tiles_n, splits, nk_all);
       const int b = j & 1;
       // warp-uniform decisions: tcgen05.ld below is executed by all 32 lanes together
-      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[b], (j >> 1) & 1))) {
+      if (!__all_sync(0xffffffffu, wait_or_stop(&acc_full[b], (j >> 1) & 1, abort_flag))) {
         if (lane == 0) atomicOr(err, 4);
-        *abort_flag = 1;
         break;
       }
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
       const int row = w.tm * kBM + q * 32 + lane;
       GemmEpilogue epz = ep;
       if (splits > 1) epz.out_f32 += (int64_t)w.z * ep.split_stride;
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN);
 #pragma unroll 1
-      for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
-        float v[32];
+      for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += kCols) {
+        float v[kCols];
         if (w.nk > 0) {
-          uint32_t r[32];
-          tmem_ld32(taddr + (uint32_t)c, r);
-#pragma unroll
-          for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(r[t]);
+          tmem_ld16(taddr + (uint32_t)c, v);
         } else {
 #pragma unroll
-          for (int t = 0; t < 32; ++t) v[t] = 0.f;  // an empty K slice contributes zero
+          for (int t = 0; t < kCols; ++t) v[t] = 0.f;  // an empty K slice contributes zero
         }
         const int col0 = w.tn * BN + c;
-        if (row < M && col0 < N) ep_apply32(epz, row, col0, N, v);
+        if (row < M && col0 < N) ep_apply(epz, row, col0, N, v);
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
@@ -421,13 +451,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
   }
 
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) {
-    // drain copies still in flight before the shared memory goes away
-    const int iss = *issued;
-    for (int kt = (iss > STAGES ? iss - STAGES : 0); kt < iss; ++kt)
-      mbar_wait(&full[kt % STAGES], (kt / STAGES) & 1);
-  }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0)
@@ -465,7 +488,8 @@ cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const GemmEp
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   const int64_t units = (int64_t)((M + kBM - 1) / kBM) * ((N + BN - 1) / BN) * splits;
-  const int grid = (int)(units < sm_count() ? units : sm_count());
+  const int slots = sm_count() * GemmSmem<BN, STAGES>::per_sm;
+  const int grid = (int)(units < slots ? units : slots);
   k_gemm_bf16_tn<BN, STAGES><<<grid, kGemmThreads, smem, s>>>(ma, mb, ep, M, N, K, splits, err);
   return cudaGetLastError();
 }
@@ -476,15 +500,20 @@ cudaError_t gemm_bf16_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat1
                          int M, int N, int K, const GemmEpilogue& ep, int32_t* err,
                          cudaStream_t s, int splits) {
   if (splits < 1 || (splits > 1 && ep.kind != kEpStoreF32)) return cudaErrorInvalidValue;
-  // 256-column tiles when they keep every SM busy and pad N no more than 128-column ones
+  // 256-column tiles when they keep every SM busy and pad N no more than
+  // 128-column ones; 64-column tiles, two CTAs per SM, when 128-column ones
+  // would not give every SM two: the epilogue is then most of the time, and
+  // twice the warps work on it (the network's products at batch 4,096, below)
   const int64_t tiles_m = (M + kBM - 1) / kBM;
   const int64_t n256 = (N + 255) / 256, n128 = (N + 127) / 128;
   const bool wide = tiles_m * n256 * splits >= sm_count() && n256 * 256 <= n128 * 128;
-  const int BN = wide ? 256 : 128;
+  const bool narrow = !wide && tiles_m * n128 * splits < 2 * sm_count();
+  const int BN = wide ? 256 : narrow ? 64 : 128;
   CUtensorMap ma, mb;
   if (!make_map_cached(&ma, A, M, K, lda, kBM)) return cudaErrorInvalidValue;
   if (!make_map_cached(&mb, B, N, K, ldb, BN)) return cudaErrorInvalidValue;
   if (wide) return launch_bn<256, 4>(ma, mb, ep, M, N, K, splits, err, s);
+  if (narrow) return launch_bn<64, 4>(ma, mb, ep, M, N, K, splits, err, s);
   return launch_bn<128, 6>(ma, mb, ep, M, N, K, splits, err, s);
 }
 

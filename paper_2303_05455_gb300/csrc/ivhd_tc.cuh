@@ -218,12 +218,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// ---- two SMs on one tile (cta_group::2) -------------------------------------
-// A cluster of two CTAs shares a 256-row tile: each holds its own 128 rows of A
-// and half of B's rows in shared memory and gets its own 128 rows of the
-// accumulator in its tensor memory; one thread of the CTA of rank 0 issues
-// the MMAs for both.
-
 // One lane of a converged warp.  The issuing warps run their loops with all
 // lanes and elect one per instruction: positions and descriptors then stay in
 // uniform registers, which the MMA and TMA instructions read; from a branch on
@@ -243,6 +237,12 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ int warp_index() {
   return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
 }
+
+// ---- two SMs on one tile (cta_group::2) -------------------------------------
+// A cluster of two CTAs shares a 256-row tile: each holds its own 128 rows of A
+// and half of B's rows in shared memory and gets its own 128 rows of the
+// accumulator in its tensor memory; one thread of the CTA of rank 0 issues
+// the MMAs for both.
 
 __device__ __forceinline__ uint32_t cta_rank() {
   uint32_t r;
