@@ -56,28 +56,39 @@ constexpr int kStepBlock = 128;      // default threads per step block (4 warps)
 
 // Default hub threshold for a graph with about `entries` symmetric row entries
 // (2 M (k + r) before mutual pairs merge): the largest power of two not above
-// entries / 70,000, within [16, 256].  A SELL slice of rows just below the
-// threshold is a chain of threshold / 8 dependent gather rounds for its warp;
-// small graphs finish in a few such chains, so a low threshold (short chains,
-// more warp-per-vertex rows) wins, while large graphs are throughput-bound and
-// lose lanes to short warp rows.  Measured best shapes: 2,000 and 70,000
-// vertices (k = 2 / 5, r = 1): 16; 1.4e6 vertices (k = 5, r = 1): 128; 64
-// embeddings with 3.7e6 vertices in total: 256.
+// entries / 70,000, within [16, 128], and 256 from 32 million entries on.  A SELL
+// slice of rows just below the threshold is a chain of threshold / 8 dependent
+// gather rounds for its warp; small graphs finish in a few such chains, so a
+// low threshold (short chains, more warp-per-vertex rows) wins, while large graphs
+// are throughput-bound and lose lanes to short warp rows.  us per step with 128 /
+// 256: 16 embeddings, 26 M entries 87.7 / 95.6; 1.4e6 vertices, k = 10, 31 M 103.2 /
+// 105.2; 3e6, k = 5, 36 M 129.8 / 127.4; 64 embeddings, 64 M 225.1 / 221.2.
+constexpr int64_t kLongSliceEntries = 32000000;
 inline int auto_hub_threshold(int64_t entries) {
+  if (entries >= kLongSliceEntries) return 256;
   int h = 16;
-  while (h < 256 && (int64_t)(2 * h) * 70000 <= entries) h *= 2;
+  while (h < 128 && (int64_t)(2 * h) * 70000 <= entries) h *= 2;
   return h;
 }
-// Rows of medium degree per warp in the warp-per-vertex region by default.
-// With the lowest hub threshold (graphs below ~2.2M symmetric entries) most
-// warp-per-vertex rows have 16-31 entries, i.e. 4-8 int4 groups for 32 lanes:
-// two rows share a warp (16 lanes each), which halves those warps and brings
-// a 70,000-vertex launch to about one wave (exact kNN graph of the
-// MNIST-shaped set: 5.9 against 6.6 us per step; 4 rows per warp 6.4 us).
-// Larger graphs keep a whole warp per row (1.4e6 points: equal within noise).
-inline int auto_vertices_per_warp(int64_t entries) {
-  return auto_hub_threshold(entries) <= 16 ? 2 : 1;
-}
+// Rows of medium degree per warp in the warp-per-vertex region by default.  Most
+// of these rows have 16 to 63 entries, i.e. 4 to 16 int4 groups for 32 lanes, so a
+// warp of its own leaves most lanes idle.  Two rows per warp (16 lanes each)
+// below a million symmetric entries, where a step is latency and shorter rows
+// per lane win (exact kNN graph of 70,000 points, us per step with 1 / 2 / 4 /
+// 8 rows: 7.14 / 5.31 / 5.42 / 5.62); four above, where it is gathers in flight
+// (exact kNN graphs: 150,000 points 11.2 / 9.1 / 8.0 / 7.6, 150,000 images 10.4 /
+// 8.7 / 7.5 / 7.9, 300,000 points 14.6 / 13.7 / 12.9 / 13.1, 300,000 with k = 10
+// and FP16 22.6 / 20.6 / 20.4 / 22.6, 600,000 26.4 / 24.5 / 24.9 / 26.3).  From
+// 1.4e6 points on (hub threshold 128: rows of 128 entries and more, which
+// keep their warps at any setting but 8) it makes no difference.
+constexpr int64_t kFourRowsEntries = 1000000;
+inline int auto_vertices_per_warp(int64_t entries) { return entries >= kFourRowsEntries ? 4 : 2; }
+
+// Grids up to this many blocks of 128 threads take k_step_ahead: about half of
+// what the GPU holds, so that the next grid fits beside it.  Measured, us per
+// step with k_step / k_step_ahead: 94 blocks 3.04 / 2.63, 314 3.56 / 3.27, 358
+// 4.36 / 3.74, 639 4.52 / 4.01, 754 4.42 / 4.40, 1,730 5.79 / 7.35.
+constexpr int kAheadBlocks = 704;
 constexpr int kMaxStepBlock = 512;   // the autotuner tries 128, 256 and 512
 constexpr int kWideRow = 512;        // rows with at least this many entries get kWideWarps warps
 constexpr int kWideWarps = 4;
@@ -173,6 +184,7 @@ struct ivhd_ctx {
   int hub_threshold = ivhd::kDefaultHubThreshold;
   int block = ivhd::kStepBlock;
   int vpw = 1;  // rows of medium degree per warp (1, 2, 4, 8)
+  int64_t vpw_entries = 0;  // > 0: vpw follows the defaults for this many symmetric entries
   bool poisoned = false;
 
   // segments (independent embeddings) and their device tables

@@ -1635,11 +1635,6 @@ int step_grid(const ivhd_ctx* ctx) {
   return (int)(nb_wide + nb_hub + nb_sell);
 }
 
-// Grids up to this many blocks of 128 threads take k_step_ahead: about half of
-// what the GPU holds, so that the next grid fits beside it.  Measured, us per
-// step with k_step / k_step_ahead: 94 blocks 3.04 / 2.63, 314 3.56 / 3.27, 358
-// 4.36 / 3.74, 639 4.52 / 4.01, 754 4.42 / 4.40, 1,730 5.79 / 7.35.
-constexpr int kAheadBlocks = 704;
 // first: the launch follows the layout's own kernels, whose writes a dependent
 // launch could not count on before its wait.
 template <int MODE, int POS, int METRIC, bool ADAPT>
