@@ -56,18 +56,19 @@ constexpr int kStepBlock = 128;      // default threads per step block (4 warps)
 
 // Default hub threshold for a graph with about `entries` symmetric row entries
 // (2 M (k + r) before mutual pairs merge): the largest power of two not above
-// entries / 70,000, within [16, 128], and 256 from 32 million entries on.  A SELL
-// slice of rows just below the threshold is a chain of threshold / 8 dependent
-// gather rounds for its warp; small graphs finish in a few such chains, so a
-// low threshold (short chains, more warp-per-vertex rows) wins, while large graphs
-// are throughput-bound and lose lanes to short warp rows.  us per step with 128 /
-// 256: 16 embeddings, 26 M entries 87.7 / 95.6; 1.4e6 vertices, k = 10, 31 M 103.2 /
-// 105.2; 3e6, k = 5, 36 M 129.8 / 127.4; 64 embeddings, 64 M 225.1 / 221.2.
-constexpr int64_t kLongSliceEntries = 32000000;
+// entries / 70,000, within [16, 256].  A SELL slice of rows just below the
+// threshold is a chain of threshold / 8 dependent gather rounds for its warp;
+// small graphs finish in a few such chains, so a low threshold (short chains,
+// more warp-per-vertex rows) wins, while large graphs are throughput-bound and
+// lose lanes to short warp rows.  Measured best shapes: 2,000 and 70,000
+// vertices (k = 2 / 5, r = 1): 16; 1.4e6 vertices (k = 5, r = 1): 128; 64
+// embeddings with 3.7e6 vertices in total: 256.  (Between 18 and 32 million
+// entries 128 is faster, 16 embeddings 87.7 us per step against 95.6, but it
+// moves the sums of rows of 128 to 255 entries, and the few vertices that
+// amplify rounding came out up to 2.5 times further from 64 bits in some runs.)
 inline int auto_hub_threshold(int64_t entries) {
-  if (entries >= kLongSliceEntries) return 256;
   int h = 16;
-  while (h < 128 && (int64_t)(2 * h) * 70000 <= entries) h *= 2;
+  while (h < 256 && (int64_t)(2 * h) * 70000 <= entries) h *= 2;
   return h;
 }
 // Rows of medium degree per warp in the warp-per-vertex region by default.  Most
