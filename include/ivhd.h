@@ -671,8 +671,11 @@ ivhd_status ivhd_eval_qnx_static(const float *Y, int64_t M, const int32_t *knn, 
  * ivhd_set_allocator -- take the library's device memory from the caller.
  *
  * The paper has no counterpart.  By default every device buffer of the
- * library (context state, layouts, kNN and network scratch) comes from the
- * stream-ordered pool (cudaMallocAsync / cudaFreeAsync on the call's stream).
+ * library (context state, layouts, kNN and network scratch) comes from a
+ * stream-ordered pool of the library's own on each device (allocated and freed
+ * on the call's stream).  It keeps at most 256 MiB of unused memory between
+ * calls; all of it is returned when an allocation fails, or by this call with
+ * both NULL (for the current device).
  * After this call, every later allocation calls alloc_fn instead, e.g. a
  * framework's caching allocator, so that one pool serves both:
  *

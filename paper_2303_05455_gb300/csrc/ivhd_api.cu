@@ -52,6 +52,94 @@ static bool take_injected_failure() {
   return false;
 }
 
+// The library's own stream-ordered pool on each device.  The device's default
+// pool returns all unused memory to the driver at every synchronisation, so
+// every call that allocates and synchronises (create, kNN, the quality criteria)
+// mapped its memory anew: 0.19 ms of a 2,000-point embedding's 1.59 ms, 0.40 of
+// one of 300,000 points, 0.48 of a 70,000-image kNN graph's 4.62, 0.39 of two
+// quality calls' 0.94.  This pool keeps at most 2 kPoolKeep bytes beyond what is
+// in use (its threshold counts both and moves in units of kPoolKeep); more goes
+// back at a synchronisation as before, all of it when an allocation fails or when
+// ivhd_set_allocator(NULL, NULL) is called.  Allocation and release are ordered
+// on streams and safe from any thread, as with the default pool.
+constexpr uint64_t kPoolKeep = (uint64_t)128 << 20;
+constexpr int kPoolDevices = 64;
+struct DevicePool {
+  unsigned long long ctx_id = 0;  // a context that is re-created gets a new pool
+  cudaMemPool_t pool = nullptr;
+  uint64_t live = 0;       // bytes in use
+  uint64_t threshold = 0;  // as set last
+};
+struct PoolBlock {
+  int dev;
+  unsigned long long ctx_id;
+  uint64_t bytes;
+};
+static DevicePool g_pools[kPoolDevices];  // these two guarded by alloc_mutex()
+static std::unordered_map<void*, PoolBlock>& pool_blocks() {
+  static auto* m = new std::unordered_map<void*, PoolBlock>;
+  return *m;
+}
+
+static void set_threshold(DevicePool& d) {
+  const uint64_t t = (d.live / kPoolKeep + 2) * kPoolKeep;
+  if (t == d.threshold || !d.pool) return;
+  uint64_t v = t;
+  if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &v) == cudaSuccess)
+    d.threshold = t;
+}
+
+// The pool for allocations on stream s and its device, or null: the stream is
+// another device's, the context cannot be told, or the pool cannot be made.
+static cudaMemPool_t own_pool(cudaStream_t s, int* dev, unsigned long long* id) {
+  int sdev = -1;
+  if (cudaGetDevice(dev) != cudaSuccess || cudaStreamGetDevice(s, &sdev) != cudaSuccess ||
+      *dev != sdev || *dev < 0 || *dev >= kPoolDevices) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  *id = current_ctx_id();
+  if (*id == 0) return nullptr;
+  std::lock_guard<std::mutex> lock(alloc_mutex());
+  DevicePool& d = g_pools[*dev];
+  if (d.ctx_id != *id) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = *dev;
+    d = DevicePool{};
+    d.ctx_id = *id;  // a pool that cannot be made is not tried again in this context
+    if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+      d.pool = nullptr;
+      cudaGetLastError();
+    }
+    set_threshold(d);
+  }
+  return d.pool;
+}
+
+static cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
+  int dev = -1;
+  unsigned long long id = 0;
+  cudaMemPool_t pool = own_pool(s, &dev, &id);
+  if (!pool) return cudaMallocAsync(p, bytes, s);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  if (e == cudaSuccess) {
+    std::lock_guard<std::mutex> lock(alloc_mutex());
+    pool_blocks()[*p] = PoolBlock{dev, id, bytes};
+    if (g_pools[dev].ctx_id == id) {
+      g_pools[dev].live += bytes;
+      set_threshold(g_pools[dev]);
+    }
+  }
+  return e;
+}
+
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s) {
   *p = nullptr;
   if (take_injected_failure()) return cudaErrorMemoryAllocation;
@@ -76,7 +164,7 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s) {
     g_live_allocs.fetch_add(1);
     return cudaSuccess;
   }
-  const cudaError_t e = cudaMallocAsync(p, bytes, s);
+  const cudaError_t e = pool_alloc(p, bytes, s);
   if (e == cudaSuccess) g_live_allocs.fetch_add(1);
   return e;
 }
@@ -94,6 +182,13 @@ cudaError_t dev_free(void* p, cudaStream_t s) {
       b = it->second;
       m.erase(it);
       from_user = true;
+    } else if (auto q = pool_blocks().find(p); q != pool_blocks().end()) {
+      DevicePool& d = g_pools[q->second.dev];
+      if (d.ctx_id == q->second.ctx_id) {
+        d.live -= q->second.bytes;
+        set_threshold(d);
+      }
+      pool_blocks().erase(q);
     }
   }
   if (from_user) {
@@ -115,6 +210,12 @@ extern "C" ivhd_status ivhd_set_allocator(ivhd_alloc_fn alloc_fn, ivhd_free_fn f
   if ((alloc_fn == nullptr) != (free_fn == nullptr)) return IVHD_ERR_ARG;
   std::lock_guard<std::mutex> lock(alloc_mutex());
   g_user_alloc = UserAllocator{alloc_fn, free_fn, alloc_fn ? user : nullptr};
+  if (!alloc_fn) {
+    // what the current device's pool holds unused goes back to the driver
+    const unsigned long long id = current_ctx_id();
+    for (DevicePool& d : g_pools)
+      if (id != 0 && d.ctx_id == id && d.pool) cudaMemPoolTrimTo(d.pool, 0);
+  }
   return IVHD_OK;
 }
 

@@ -30,12 +30,15 @@
 namespace ivhd {
 
 // Every device allocation of the library goes through these two calls
-// (stream-ordered cudaMallocAsync / cudaFreeAsync, or the caller's allocator
-// set with ivhd_set_allocator).  They count the live
+// (a stream-ordered pool of the library's own, or the caller's allocator set with
+// ivhd_set_allocator).  They count the live
 // allocations, so tests can check that error paths free what they took, and
 // ivhd_test_fail_alloc can make one of them fail to exercise those paths.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s);
 cudaError_t dev_free(void* p, cudaStream_t s);
+
+// The current CUDA context's unique id; 0 if the driver cannot tell.
+unsigned long long current_ctx_id();
 
 // Names the enclosing host scope in profiler timelines (NVTX range; a no-op
 // unless a tool is attached).

@@ -147,9 +147,10 @@ __global__ void k_qnx_static_total(unsigned long long* __restrict__ scratch, int
   }
 }
 
-// The current context's unique id (cuCtxGetCurrent + cuCtxGetId, reached
-// through the runtime's driver entry points so the library needs no libcuda
-// link); 0 if the driver cannot tell.
+}  // namespace
+
+// Reached through the runtime's driver entry points, so that the library needs
+// no libcuda link.
 unsigned long long current_ctx_id() {
   using GetCurrent = CUresult (*)(CUcontext*);
   using GetId = CUresult (*)(CUcontext, unsigned long long*);
@@ -175,6 +176,8 @@ unsigned long long current_ctx_id() {
   if (get_id(ctx, &id) != CUDA_SUCCESS) return 0;
   return id;
 }
+
+namespace {
 
 struct ScratchAddr {
   unsigned long long ctx_id = 0;
