@@ -448,71 +448,116 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
 // ---- operand preparation ---------------------------------------------------
 
-// FP32: A = [hi | hi | lo], B = [hi | lo | hi] along K (3N, zero-padded to Kp);
-// either output may be null (queries fill A, the base set B).
-__global__ void k_prep_f32(const float* __restrict__ X, int64_t M, int N, int Kp,
-                           __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= M * Kp) return;
-  const int64_t i = e / Kp;
-  const int c = (int)(e - i * Kp);
-  const int seg = c / N, d = c - seg * N;
-  __nv_bfloat16 a = __float2bfloat16_rn(0.f), b = a;
-  if (seg < 3) {
-    const float x = X[i * N + d];
-    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-    a = (seg == 2) ? lo : hi;
-    b = (seg == 1) ? lo : hi;
-  }
-  if (A) A[e] = a;
-  if (B) B[e] = b;
+// Both kernels write a row's operands and its norm from one read of it, a warp
+// per row over a resident grid.  uint8 is bound by the operands' stores, float by
+// the FP64 sums (504 MB would take 74 us): 300,000 x 100 floats 476 -> 259 us (a thread per element, and a thread per row for the
+// norms), 70,000 x 784 bytes 248 -> 33 us.
+constexpr int kPrepWarps = 8;
+inline unsigned prep_blocks(int64_t M, int sms) {
+  const int64_t all = (M + kPrepWarps - 1) / kPrepWarps, resident = (int64_t)sms * 8;
+  return (unsigned)(all < resident ? all : resident);
 }
 
-// FP32 norms (FP64 sum, rounded once); the largest goes to nrm[M], which
-// starts at zero (norms are not negative, so their bits order as integers).
-__global__ void k_norms_f32(const float* __restrict__ X, int64_t M, int N, float* __restrict__ nrm) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float n = 0.f;
-  if (i < M) {
-    double s = 0.0;
-    for (int d = 0; d < N; ++d) {
-      const double x = X[i * N + d];
-      s += x * x;
+// FP32: A = [hi | hi | lo], B = [hi | lo | hi] along K (3N, zero-padded to Kp);
+// either output may be null (queries fill A, the base set B).  Norms: an FP64 sum,
+// rounded once; the largest goes to nrm[M], which starts at zero (norms are not
+// negative, so their bits order as integers).
+// V: features per access; 4 needs N % 4 == 0 and X on 16 bytes, then every part of
+// an operand row starts on 8 (Kp is a multiple of 64).
+template <int V>
+__global__ void k_prep_f32(const float* __restrict__ X, int64_t M, int N, int Kp,
+                           __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
+                           float* __restrict__ nrm) {
+  struct __align__(2 * V) Part {
+    __nv_bfloat16 v[V];
+  };
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * kPrepWarps;
+  unsigned top = 0;
+  for (int64_t i = (int64_t)blockIdx.x * kPrepWarps + (threadIdx.x >> 5); i < M; i += warps) {
+    __nv_bfloat16* a = A ? A + i * Kp : nullptr;
+    __nv_bfloat16* b = B ? B + i * Kp : nullptr;
+    double sum = 0.0;
+    for (int d = lane * V; d < N; d += 32 * V) {
+      float x[V];
+      if constexpr (V == 4) {
+        const float4 w = *reinterpret_cast<const float4*>(X + i * N + d);
+        x[0] = w.x, x[1] = w.y, x[2] = w.z, x[3] = w.w;
+      } else {
+        x[0] = X[i * N + d];
+      }
+      Part hi, lo;
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        hi.v[u] = __float2bfloat16_rn(x[u]);
+        lo.v[u] = __float2bfloat16_rn(x[u] - __bfloat162float(hi.v[u]));
+        sum += (double)x[u] * (double)x[u];
+      }
+      if (a) {
+        *reinterpret_cast<Part*>(a + d) = hi;
+        *reinterpret_cast<Part*>(a + N + d) = hi;
+        *reinterpret_cast<Part*>(a + 2 * N + d) = lo;
+      }
+      if (b) {
+        *reinterpret_cast<Part*>(b + d) = hi;
+        *reinterpret_cast<Part*>(b + N + d) = lo;
+        *reinterpret_cast<Part*>(b + 2 * N + d) = hi;
+      }
     }
-    n = (float)s;
-    nrm[i] = n;
+    for (int c = 3 * N + lane; c < Kp; c += 32) {
+      if (a) a[c] = __float2bfloat16_rn(0.f);
+      if (b) b[c] = __float2bfloat16_rn(0.f);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    const float n = (float)sum;
+    if (lane == 0) nrm[i] = n;
+    top = max(top, __float_as_uint(n));
   }
-  const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(n));
-  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned*>(nrm + M), top);
+  if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(nrm + M), top);
 }
 
 // uint8: A = B = x - 128 (zero-padded to Kp); norms of the shifted rows.
+// Eight columns per lane and store; V: bytes per load (8 needs N % 8 == 0 and X on 8).
+template <int V>
 __global__ void k_prep_u8(const uint8_t* __restrict__ X, int64_t M, int N, int Kp,
-                          __nv_bfloat16* __restrict__ A) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= M * Kp) return;
-  const int64_t i = e / Kp;
-  const int c = (int)(e - i * Kp);
-  A[e] = __float2bfloat16_rn(c < N ? (float)X[i * N + c] - 128.f : 0.f);
-}
-
-__global__ void k_norms_u8s(const uint8_t* __restrict__ X, int64_t M, int N,
-                            int32_t* __restrict__ nrm) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M) return;
-  int32_t s = 0;
-  for (int d = 0; d < N; ++d) {
-    const int32_t v = (int32_t)X[i * N + d] - 128;
-    s += v * v;
+                          __nv_bfloat16* __restrict__ A, int32_t* __restrict__ nrm) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * kPrepWarps;
+  for (int64_t i = (int64_t)blockIdx.x * kPrepWarps + (threadIdx.x >> 5); i < M; i += warps) {
+    const uint8_t* x = X + i * N;
+    int32_t sum = 0;
+    for (int c = lane * 8; c < Kp; c += 256) {
+      uint8_t t[8];
+      if constexpr (V == 8) {
+        uint2 w = make_uint2(0x80808080u, 0x80808080u);  // 128: the shifted value is 0
+        if (c < N) w = *reinterpret_cast<const uint2*>(x + c);
+        memcpy(t, &w, 8);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u] = c + u < N ? x[c + u] : 128;
+      }
+      __nv_bfloat16 o[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int v = (int)t[u] - 128;
+        o[u] = __float2bfloat16_rn((float)v);
+        sum += v * v;
+      }
+      uint4 w;
+      memcpy(&w, o, 16);
+      *reinterpret_cast<uint4*>(A + i * Kp + c) = w;
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) nrm[i] = sum;
   }
-  nrm[i] = s;
 }
 
 // ---- FP32 re-rank and certificate (warp per row, lane = candidate) --------
 
-__device__ __forceinline__ void cas(float& d, int& j, int lane, int mask, bool up) {
-  const float od = __shfl_xor_sync(0xffffffffu, d, mask);
+template <class D>
+__device__ __forceinline__ void cas(D& d, int& j, int lane, int mask, bool up) {
+  const D od = __shfl_xor_sync(0xffffffffu, d, mask);
   const int oj = __shfl_xor_sync(0xffffffffu, j, mask);
   const bool lower = (lane & mask) == 0;
   // the lower lane keeps the smaller pair when sorting up
@@ -554,18 +599,21 @@ __device__ __forceinline__ float chain_dist(const float* __restrict__ xi,
   return acc;
 }
 
-// Bitonic sort of one (d, j) pair per lane across the warp, ascending.
-__device__ __forceinline__ void warp_sort(float& d, int& j, int lane) {
+// Bitonic sort of one (d, j) pair per lane across the warp, ascending.  SORTED:
+// lanes already in sorted runs of this length, every other one descending.
+template <int SORTED = 1, class D>
+__device__ __forceinline__ void warp_sort(D& d, int& j, int lane) {
 #pragma unroll
-  for (int kk = 2; kk <= 32; kk <<= 1)
+  for (int kk = 2 * SORTED; kk <= 32; kk <<= 1)
 #pragma unroll
     for (int m = kk >> 1; m > 0; m >>= 1) cas(d, j, lane, m, (lane & kk) == 0);
 }
 
 // The 32 smallest of a warp's sorted (d, j) and the sorted (dn, jn): the first
 // against the second reversed is bitonic, and a bitonic merge sorts it.
-__device__ __forceinline__ void warp_merge(float& d, int& j, float dn, int jn, int lane) {
-  const float rd = __shfl_sync(0xffffffffu, dn, 31 - lane);
+template <class D>
+__device__ __forceinline__ void warp_merge(D& d, int& j, D dn, int jn, int lane) {
+  const D rd = __shfl_sync(0xffffffffu, dn, 31 - lane);
   const int rj = __shfl_sync(0xffffffffu, jn, 31 - lane);
   if (better(rd, rj, d, j)) {
     d = rd;
@@ -682,27 +730,39 @@ __global__ void k_rerank(const float* __restrict__ Q, int Mq, const float* __res
 }
 
 // uint8: the n_lists exact lists of each row (ascending by (distance, index))
-// merged into the k nearest.
+// merged into the k <= 32 nearest: a warp per row, 32 / L lists per pass, every
+// other one read backwards as the sort wants it; a pass without a candidate
+// before the k-th so far is skipped (10,000 queries, 34 lists of 8: 41 -> 16 us;
+// 70,000 rows, 6 lists: 26 -> 27; a thread per row left most of the chip idle).
 template <int L>
 __global__ void k_merge_u8(const int32_t* __restrict__ ids, const int32_t* __restrict__ keys,
                            int64_t M, int k, int n_lists, int32_t* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31, n = n_lists * L;
+  const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= M) return;
-  const int32_t* ja = ids + i * n_lists * L;
-  const int32_t* da = keys + i * n_lists * L;
-  int head[2 * kMaxKnnSegments];
-  for (int h = 0; h < n_lists; ++h) head[h] = 0;
-  for (int q = 0; q < k; ++q) {
-    int bh = -1;
-    for (int h = 0; h < n_lists; ++h) {
-      if (head[h] >= L) continue;
-      const int64_t a = (int64_t)h * L + head[h];
-      const int64_t b = (int64_t)bh * L + (bh < 0 ? 0 : head[bh]);
-      if (bh < 0 || better(da[a], ja[a], da[b], ja[b])) bh = h;
+  // (one list per pass, L = 32: ascending, nothing to sort)
+  const int from = (L < 32 && (lane & L)) ? (lane ^ (L - 1)) : lane;
+  int32_t d = INT_MAX, j = INT_MAX;
+  for (int at0 = 0; at0 < n; at0 += 32) {
+    int32_t dc = INT_MAX, jc = INT_MAX;
+    if (at0 + from < n) {
+      dc = keys[i * n + at0 + from];
+      jc = ids[i * n + at0 + from];
     }
-    out[i * k + q] = ja[(int64_t)bh * L + head[bh]];
-    ++head[bh];
+    if (at0 > 0) {
+      const int32_t dk = __shfl_sync(0xffffffffu, d, k - 1);
+      const int32_t jk = __shfl_sync(0xffffffffu, j, k - 1);
+      if (!__any_sync(0xffffffffu, better(dc, jc, dk, jk))) continue;
+    }
+    warp_sort<L>(dc, jc, lane);
+    if (at0 == 0) {
+      d = dc;
+      j = jc;
+    } else {
+      warp_merge(d, j, dc, jc, lane);
+    }
   }
+  if (lane < k) out[i * k + lane] = j;
 }
 
 template <bool U8, int L>
@@ -779,26 +839,46 @@ int knn_tc_kp(int32_t dtype, int32_t N) {
   return (int)(((K + kBK - 1) / kBK) * kBK);
 }
 
-// The M norms and, at nrm[M], the largest of them.
-static cudaError_t row_norms_f32(const float* X, int64_t M, int N, float* nrm, cudaStream_t s) {
+static int sm_count() {
+  int sms = 0, dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess &&
+                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
+             ? sms
+             : 0;
+}
+
+// The M x Kp operands (either may be null), the M norms and, at nrm[M], the
+// largest of them.
+static cudaError_t prep_f32(const float* X, int64_t M, int N, __nv_bfloat16* A, __nv_bfloat16* B,
+                            float* nrm, int sms, cudaStream_t s) {
   const cudaError_t e = cudaMemsetAsync(nrm + M, 0, sizeof(float), s);
   if (e != cudaSuccess) return e;
-  k_norms_f32<<<(unsigned)((M + 255) / 256), 256, 0, s>>>(X, M, N, nrm);
+  const int Kp = knn_tc_kp(IVHD_KNN_F32, N);
+  const unsigned g = prep_blocks(M, sms);
+  if (N % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0)
+    k_prep_f32<4><<<g, 32 * kPrepWarps, 0, s>>>(X, M, N, Kp, A, B, nrm);
+  else
+    k_prep_f32<1><<<g, 32 * kPrepWarps, 0, s>>>(X, M, N, Kp, A, B, nrm);
+  return cudaGetLastError();
+}
+
+static cudaError_t prep_u8(const uint8_t* X, int64_t M, int N, __nv_bfloat16* A, int32_t* nrm,
+                           int sms, cudaStream_t s) {
+  const int Kp = knn_tc_kp(IVHD_KNN_U8, N);
+  const unsigned g = prep_blocks(M, sms);
+  if (N % 8 == 0 && (reinterpret_cast<uintptr_t>(X) & 7) == 0)
+    k_prep_u8<8><<<g, 32 * kPrepWarps, 0, s>>>(X, M, N, Kp, A, nrm);
+  else
+    k_prep_u8<1><<<g, 32 * kPrepWarps, 0, s>>>(X, M, N, Kp, A, nrm);
   return cudaGetLastError();
 }
 
 cudaError_t knn_tc_prepare_base(const void* X, int32_t dtype, int64_t M, int32_t N,
                                 __nv_bfloat16* B, void* nrm, cudaStream_t s) {
-  const int Kp = knn_tc_kp(dtype, N);
-  auto blocks = [](int64_t n) { return (unsigned)((n + 255) / 256); };
-  if (dtype == IVHD_KNN_U8) {
-    k_prep_u8<<<blocks(M * Kp), 256, 0, s>>>((const uint8_t*)X, M, N, Kp, B);
-    k_norms_u8s<<<blocks(M), 256, 0, s>>>((const uint8_t*)X, M, N, (int32_t*)nrm);
-  } else {
-    k_prep_f32<<<blocks(M * Kp), 256, 0, s>>>((const float*)X, M, N, Kp, nullptr, B);
-    return row_norms_f32((const float*)X, M, N, (float*)nrm, s);
-  }
-  return cudaGetLastError();
+  const int sms = sm_count();
+  if (sms == 0) return cudaErrorInvalidDevice;
+  if (dtype == IVHD_KNN_U8) return prep_u8((const uint8_t*)X, M, N, B, (int32_t*)nrm, sms, s);
+  return prep_f32((const float*)X, M, N, nullptr, B, (float*)nrm, sms, s);
 }
 
 ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
@@ -819,7 +899,6 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
   cudaError_t e = cudaMemsetAsync(err, 0, 8 * sizeof(int32_t), s);
   int32_t* n_fb = err + 1;
   int32_t* maxerr_bits = err + 2;
-  auto blocks = [](int64_t n) { return (unsigned)((n + 255) / 256); };
   CUtensorMap ma, mb;
   if (!make_map(&ma, A, Mq, Kp, Kp, kTM) || !make_map(&mb, B, M, Kp, Kp, kTN / 2))
     return IVHD_ERR_CUDA;
@@ -829,10 +908,8 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
   // minimises waves x (tiles per segment + a fixed cost of about two tiles per
   // CTA); a segment keeps at least 4 tiles of 256 columns.  Each segment
   // yields its own lists, merged per row afterwards.
-  int sms = 0, dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return IVHD_ERR_CUDA;
+  const int sms = sm_count();
+  if (sms == 0) return IVHD_ERR_CUDA;
   const int64_t row_blocks = 2 * ((Mq + 2 * kTM - 1) / (2 * kTM));
   const int all_tiles = (int)((M + kTN - 1) / kTN);
   int want = 1;
@@ -856,16 +933,10 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
     int32_t* lkeys = b.get<int32_t>(Mq * n_lists * L);
     if (!b.ok) return IVHD_ERR_OOM;
     if (e == cudaSuccess) {
-      const uint8_t* X = (const uint8_t*)P.X;
-      const uint8_t* Q = (const uint8_t*)P.Q;
-      if (!base) {
-        k_prep_u8<<<blocks(M * Kp), 256, 0, s>>>(X, M, N, Kp, B);
-        k_norms_u8s<<<blocks(M), 256, 0, s>>>(X, M, N, nrm);
-      }
-      if (!P.self) {
-        k_prep_u8<<<blocks(Mq * Kp), 256, 0, s>>>(Q, Mq, N, Kp, A);
-        k_norms_u8s<<<blocks(Mq), 256, 0, s>>>(Q, Mq, N, qnrm);
-      }
+      if (!base) e = prep_u8((const uint8_t*)P.X, M, N, B, nrm, sms, s);
+      if (!P.self && e == cudaSuccess) e = prep_u8((const uint8_t*)P.Q, Mq, N, A, qnrm, sms, s);
+    }
+    if (e == cudaSuccess) {
       e = (L == 8) ? launch_tc<true, 8>(ma, mb, nullptr, nrm, nullptr, qnrm, (int)Mq, (int)M, Kp,
                                         P.self, k, segs, seg_tiles, 0.f, bounds, lids, (float*)lkeys, err,
                                         s)
@@ -874,10 +945,11 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
                                                (float*)lkeys, err, s);
     }
     if (e == cudaSuccess) {
+      const unsigned g8 = (unsigned)((Mq + 7) / 8);
       if (L == 8)
-        k_merge_u8<8><<<blocks(Mq), 256, 0, s>>>(lids, lkeys, Mq, k, n_lists, out_knn);
+        k_merge_u8<8><<<g8, 256, 0, s>>>(lids, lkeys, Mq, k, n_lists, out_knn);
       else
-        k_merge_u8<kKnnList><<<blocks(Mq), 256, 0, s>>>(lids, lkeys, Mq, k, n_lists, out_knn);
+        k_merge_u8<kKnnList><<<g8, 256, 0, s>>>(lids, lkeys, Mq, k, n_lists, out_knn);
       e = cudaGetLastError();
     }
   } else {
@@ -892,13 +964,11 @@ ivhd_status knn_tc_build(const KnnProblem& P, int32_t* out_knn, cudaStream_t s,
     const float* Q = (const float*)P.Q;
     if (e == cudaSuccess) {
       if (P.self) {
-        k_prep_f32<<<blocks(M * Kp), 256, 0, s>>>(X, M, N, Kp, A, B);
+        e = prep_f32(X, M, N, A, B, nrm, sms, s);
       } else {
-        if (!base) k_prep_f32<<<blocks(M * Kp), 256, 0, s>>>(X, M, N, Kp, nullptr, B);
-        k_prep_f32<<<blocks(Mq * Kp), 256, 0, s>>>(Q, Mq, N, Kp, A, nullptr);
-        e = row_norms_f32(Q, Mq, N, qnrm, s);
+        if (!base) e = prep_f32(X, M, N, nullptr, B, nrm, sms, s);
+        if (e == cudaSuccess) e = prep_f32(Q, Mq, N, A, nullptr, qnrm, sms, s);
       }
-      if (!base && e == cudaSuccess) e = row_norms_f32(X, M, N, nrm, s);
     }
     if (e == cudaSuccess) {
       e = (L == 16) ? launch_tc<false, 16>(ma, mb, nrm, nullptr, qnrm, nullptr, (int)Mq, (int)M,
