@@ -116,7 +116,8 @@ typedef struct {
                              2: a cluster of 8 blocks, each with a full copy of the
                              positions, updated through distributed shared memory;
                              1: a single block; 0 (default): the cluster for graphs of at
-                             most 40,000 stored entries, where it is faster, else one
+                             most 40,000 stored entries, where it is faster (a wait that
+                             expires leaves NaN positions, see ivhd_stress), else one
                              launch per step; -1: always one launch per step;
                              3: a persistent cooperative grid of any size (FP32 gathers,
                              no adaptive b, else IVHD_ERR_ARG): every block stays
@@ -130,11 +131,11 @@ typedef struct {
     int32_t vertices_per_warp; /* warp-per-vertex rows of medium degree processed several
                              to a warp: 1, 2, 4 or 8 rows per warp, each on 32 / that many
                              lanes, for the rows below 512 / that many entries (longer rows
-                             keep a whole warp); 0 = library default: 1 (a whole warp per
-                             row).  Measured (us per step, hub threshold / rows per warp):
-                             random 200,000-vertex graph with hubs 16/4 11.0 against 12.0
-                             for the best shape with 1; no gain on the exact kNN graphs of
-                             70,000 and 1.4e6 points.  ivhd_autotune searches it */
+                             keep a whole warp); 0 = library default: 2 below a million
+                             symmetric entries, 4 above.  Measured (us per step with
+                             1 / 2 / 4 / 8): exact kNN graphs of 70,000 points 7.14 /
+                             5.31 / 5.42 / 5.62, of 300,000 points 14.6 / 13.7 / 12.9 /
+                             13.1.  ivhd_autotune searches it */
     int32_t order;        /* vertex order of the layout (ivhd_order); default
                              IVHD_ORDER_DEGREE */
     void *stream;         /* cudaStream_t for all work of the context; NULL = default stream */

@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // cores, set the time (whole build, 300,000 x 100 floats, k = 5: 70.4 -> 44.2 ms
     // with queues, 42.7 with appends that do not branch, loads that run ahead and
     // shared bounds, 38.8 with the second producer; 70,000 x 784 bytes 6.00 ->
-    // 5.59 -> 5.01 -> 4.44 ms).
+    // 5.59 -> 5.01 -> 4.44 ms; 38.4 and 4.24 since the operands are prepared in
+    // one pass).
     // uint8: the float key and the float threshold are within 2 of the exact
     // integers (magnitudes below 2^26), so the test allows 16 and the queue takes
     // the exact keys.

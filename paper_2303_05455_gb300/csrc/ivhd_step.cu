@@ -1269,7 +1269,7 @@ static size_t resident_bytes(const ivhd_ctx* ctx, bool with_ids) {
 // read through L1; 2: ids in shared memory too; 4: persistent grid (resident = 3).
 // 3: thread-block cluster (resident = 2, or automatically for graphs of at
 // most kClusterAutoEntries stored entries, where it measured faster than one
-// launch per step: 2,000-4,000 vertices 2.0-2.5 us against 3.1-3.4 us per step;
+// launch per step: 2,000-4,000 vertices 1.2-2.1 us against 2.6-3.3 us per step;
 // at 5,000 vertices with hubs it was slower).
 constexpr int64_t kClusterAutoEntries = 40000;
 int resident_mode(const ivhd_ctx* ctx) {
