@@ -343,6 +343,10 @@ __global__ void __launch_bounds__(kGemmThreads, GemmSmem<BN, STAGES>::per_sm)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
+  // What precedes in the stream is complete from here on.  The next kernel may be
+  // launched once every CTA is here: each holds its tensor memory by then, so a
+  // waiting CTA of the next kernel cannot keep it from one of this kernel.
+  depend();
 
   if (warp == 0 || warp == 2 + kEpiWarps) {
     // TMA producers, one for each operand (one warp's copies reach about 50
@@ -475,7 +479,7 @@ int sm_count() {
 
 template <int BN, int STAGES>
 cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const GemmEpilogue& ep, int M,
-                      int N, int K, int splits, int32_t* err, cudaStream_t s) {
+                      int N, int K, int splits, int32_t* err, cudaStream_t s, bool dependent) {
   const int smem = GemmSmem<BN, STAGES>::total;
   static bool attr_set[64] = {};  // one attribute call per instantiation and device
   int dev = 0;
@@ -489,15 +493,15 @@ cudaError_t launch_bn(const CUtensorMap& ma, const CUtensorMap& mb, const GemmEp
   const int64_t units = (int64_t)((M + kBM - 1) / kBM) * ((N + BN - 1) / BN) * splits;
   const int slots = sm_count() * GemmSmem<BN, STAGES>::per_sm;
   const int grid = (int)(units < slots ? units : slots);
-  k_gemm_bf16_tn<BN, STAGES><<<grid, kGemmThreads, smem, s>>>(ma, mb, ep, M, N, K, splits, err);
-  return cudaGetLastError();
+  return launch_dependent(dependent, k_gemm_bf16_tn<BN, STAGES>, dim3(grid), dim3(kGemmThreads),
+                          smem, s, ma, mb, ep, M, N, K, splits, err);
 }
 
 }  // namespace
 
 cudaError_t gemm_bf16_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb,
                          int M, int N, int K, const GemmEpilogue& ep, int32_t* err,
-                         cudaStream_t s, int splits) {
+                         cudaStream_t s, int splits, bool dependent) {
   if (splits < 1 || (splits > 1 && ep.kind != kEpStoreF32)) return cudaErrorInvalidValue;
   // 256-column tiles when they keep every SM busy and pad N no more than
   // 128-column ones; 64-column tiles, two CTAs per SM, when 128-column ones
@@ -511,9 +515,9 @@ cudaError_t gemm_bf16_tn(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat1
   CUtensorMap ma, mb;
   if (!make_map_cached(&ma, A, M, K, lda, kBM)) return cudaErrorInvalidValue;
   if (!make_map_cached(&mb, B, N, K, ldb, BN)) return cudaErrorInvalidValue;
-  if (wide) return launch_bn<256, 4>(ma, mb, ep, M, N, K, splits, err, s);
-  if (narrow) return launch_bn<64, 4>(ma, mb, ep, M, N, K, splits, err, s);
-  return launch_bn<128, 6>(ma, mb, ep, M, N, K, splits, err, s);
+  if (wide) return launch_bn<256, 4>(ma, mb, ep, M, N, K, splits, err, s, dependent);
+  if (narrow) return launch_bn<64, 4>(ma, mb, ep, M, N, K, splits, err, s, dependent);
+  return launch_bn<128, 6>(ma, mb, ep, M, N, K, splits, err, s, dependent);
 }
 
 // out[i] = sum_z part[z * stride + i] over `splits` slices in order (deterministic).
