@@ -114,9 +114,14 @@ __device__ __forceinline__ bool row_ok(int64_t beg, int64_t end, int64_t n_slots
   atomicAdd(&g_check_violations, 1ull);
   return false;
 }
+// Indices that were skipped when their row was read and are skipped again.
+__device__ __forceinline__ void skipped_again(int n) {
+  if (n) atomicAdd(&g_check_violations, (unsigned long long)n);
+}
 #else
 __device__ __forceinline__ constexpr bool index_ok(uint32_t, uint32_t) { return true; }
 __device__ __forceinline__ constexpr bool row_ok(int64_t, int64_t, int64_t) { return true; }
+__device__ __forceinline__ constexpr void skipped_again(int) {}
 #endif
 
 // Warp w of the warp-per-vertex region (the hub rows, in descending degree):
@@ -1097,7 +1102,7 @@ __global__ void __launch_bounds__(HELD ? kHeldThreads : kResidentThreads, 1)
     ClusterRow R{nullptr, 0, 0, 32, 0, false};
     uint32_t e[kHeld];
     uint32_t any_rn = 0;
-    int groups = 0;
+    int groups = 0, bad = 0;  // bad: held entries outside the graph (checked builds)
     float2 v = make_float2(0.f, 0.f), ex = v;
     if (busy) {
       R = cluster_row(A, item, lane);
@@ -1114,7 +1119,9 @@ __global__ void __launch_bounds__(HELD ? kHeldThreads : kResidentThreads, 1)
 #pragma unroll
       for (int q = 0; q < kHeld; ++q) {
         // padding gathers the row's own position as an nn term: u = 0, no force
-        if (e[q] == kPad || !index_ok(e[q] & kIdxMask, (uint32_t)M)) e[q] = (uint32_t)R.p;
+        const bool skip = e[q] != kPad && !index_ok(e[q] & kIdxMask, (uint32_t)M);
+        bad += skip;
+        if (e[q] == kPad || skip) e[q] = (uint32_t)R.p;
         any_rn |= (uint32_t)(__any_sync(0xffffffffu, (e[q] & kRnBit) != 0)) << q;
       }
       if (R.own) {
@@ -1134,6 +1141,7 @@ __global__ void __launch_bounds__(HELD ? kHeldThreads : kResidentThreads, 1)
                      "r"((uint32_t)M * 8u)
                      : "memory");
       if (busy) {
+        if (it > 0) skipped_again(bad);
         const float2* src = (it & 1) ? ys1 : ys0;
         float fx = 0.f, fy = 0.f;
         if (groups == 2)
